@@ -84,12 +84,16 @@ double item_cost(const Grid& g, int pass) {
 int thread_class(int t) { return t <= 128 ? 128 : (t <= 256 ? 256 : 512); }
 
 // One launch of a stage: pass kind (0 = A, 1 = B, 2 = C), z group of pass B,
-// block size, and its slice of the item array.
+// block size, and its slice of the item array (threads and smem of a general
+// pass-B launch are in `bl`).
 struct Launch {
   int kind, group, threads;
   int off, cnt;
   size_t smem;
   int warp = -1;   // >= 0: the warp-engine launch of this pass for descriptor `warp`
+  bool general = false;   // pass B on the general warp kernel (passb_g.cuh), one CTA per item
+  PassBG bg{};
+  PassBGLaunch bl{};
   Grid g{};        // its grid
   int R = 1;       // its ky classes (pass B)
 };
@@ -218,9 +222,9 @@ BatchInst make_inst(const Member& m, unsigned* red, double h, int relax) {
   I.d.plan_ly = c->plan_ly;
   I.d.R = 1;
   I.d.ks = 0;
+  I.d.tw_wy = c->d_tw_wy;
   if (warp_member(c)) {   // the warp passes' tables and ky classes
     I.d.R = c->R;
-    I.d.tw_wy = c->d_tw_wy;
     I.d.tw_wx = c->d_tw_wx;
     I.d.tw_wx2 = c->d_tw_wx2;
     I.d.err = c->d_flag;
@@ -252,12 +256,27 @@ int build_list(mmp_batch* b, const std::vector<int>& mem) {
   L.members = mem;
   std::map<std::tuple<int, int, int>, std::vector<std::pair<double, BatchItem>>> sec;
   std::map<std::tuple<int, int, int>, size_t> smem;
+  std::map<std::tuple<int, int, int>, Launch> general;   // pass B sections of the general warp kernel
   std::vector<Launch> warp;   // the warp-engine members' launches
   for (int k = 0; k < (int)mem.size(); ++k) {
     const mmp_ctx* c = b->members[mem[k]].ctx;
     const Grid& g = c->g;
-    if (warp_member(c)) {
+    const bool wm = warp_member(c);
+    // pass B on the general warp kernel: one launch per nz and y length
+    PassBG bg;
+    const bool gb = passb_g_use(g, wm ? c->R : 1, wm) && passb_g_shape(g, &bg);
+    if (gb) {
+      const auto key = std::make_tuple(1, 1000 + g.nz, bg.Q * 32 * bg.M);
+      Launch& l = general[key];
+      l.general = true;
+      l.g = g;
+      l.bg = bg;
+      l.bl = passb_g_plan(g, bg, 0);
+      for (int kx = 0; kx < g.kxn; kx += l.bl.kp) sec[key].push_back({item_cost(g, 1), BatchItem{k, kx, 0}});
+    }
+    if (wm) {
       for (int kind = 0; kind < 3; ++kind) {
+        if (kind == 1 && gb) continue;
         Launch l{};
         l.kind = kind;
         l.warp = k;
@@ -273,19 +292,21 @@ int build_list(mmp_batch* b, const std::vector<int>& mem) {
     const auto kb = std::make_tuple(1, nz_group(g.nz), thread_class(c->thrB));
     const auto kc = std::make_tuple(2, 0, thread_class(c->thrC));
     smem[ka] = std::max(smem[ka], smem_a(g));
-    smem[kb] = std::max(smem[kb], smem_b(g));
+    if (!gb) smem[kb] = std::max(smem[kb], smem_b(g));
     smem[kc] = std::max(smem[kc], smem_c(g));
     for (int z = 0; z < g.nz; ++z) {
       for (int t = 0; t < tiles; ++t) sec[ka].push_back({item_cost(g, 0), BatchItem{k, t, z}});
       for (int t = 0; t < tiles_c; ++t) sec[kc].push_back({item_cost(g, 2), BatchItem{k, t, z}});
     }
-    for (int kx = 0; kx < g.kxn; ++kx) sec[kb].push_back({item_cost(g, 1), BatchItem{k, kx, 0}});
+    for (int kx = 0; !gb && kx < g.kxn; ++kx) sec[kb].push_back({item_cost(g, 1), BatchItem{k, kx, 0}});
   }
   std::vector<BatchItem> items;
   for (auto& kv : sec) {   // std::map order: kind, then group, then block size
     auto& v = kv.second;
     std::stable_sort(v.begin(), v.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
     Launch l;
+    const auto gl = general.find(kv.first);
+    if (gl != general.end()) l = gl->second;
     l.kind = std::get<0>(kv.first);
     l.group = std::get<1>(kv.first);
     l.threads = std::get<2>(kv.first);
@@ -351,6 +372,7 @@ cudaError_t launch_one(mmp_batch* b, const Launch& l, int stage, cudaStream_t s)
   if (l.warp >= 0) return launch_batch_warp(l.kind, b->d_inst, l.warp, l.g, l.R, stage, s);
   const BatchItem* it = b->d_items + l.off;
   if (l.kind == 0) return launch_batch_passA(b->d_inst, it, l.cnt, stage, l.threads, l.smem, s);
+  if (l.general) return launch_passB_g(l.g, DemagArgs{}, l.bg, l.bl, l.cnt, b->d_inst, it, s);
   if (l.kind == 1) return launch_batch_passB(l.group, b->d_inst, it, l.cnt, l.threads, l.smem, s);
   return launch_batch_field(b->d_inst, it, l.cnt, stage, l.threads, l.smem, s);
 }

@@ -84,13 +84,14 @@ struct DemagArgs {
   int R;                     // residue classes of ky per cluster
   int ks;                    // pass B stages the kernel slice in shared memory
   // warp engine (wfft.cuh): twiddle tables w_N^(l k1) at [k1 * 32 + l]
-  const float2* tw_wy;       // N = Ly (pass B)
+  const float2* tw_wy;       // N = Ly (pass B; the general pass B: Py / Q)
   const float2* tw_wx;       // N = Px / 2 (passes A and C)
   const float2* tw_wx2;      // w_Px^x, x < Px / 2 (natural order; passes A and C)
   const float* tw_tc;        // tensor-core DFT32 matrices, split TF32 (tcdft.cuh layout)
   unsigned* err;             // set to 1 by a device wait that ran past its limit
-  int engine;                // pass B: 0 block Stockham passes, 1 warp passes, 2 warp passes with
-                             // the final DFT32 of each y transform on the tensor cores
+  int engine;                // pass B: 0 block engine, 1 warp passes, 2 warp passes with the final
+                             // DFT32 of each y transform on the tensor cores; 0 and 1 run the
+                             // general warp pass B where passb_g_use says so
 };
 
 struct Coefs {
@@ -169,6 +170,32 @@ inline bool passb_w_supported(const Grid& g, int R) {
   if (g.ny > Ly) return false;
   return g.nz == 1 || g.nz == 2 || g.nz == 4 || g.nz == 8;
 }
+// General warp pass B (passb_g.cuh): half z length H (padded 2 H), y length
+// Py = Q * 32 M.  False when the grid is outside it: nz > 8, a padded y length
+// that is not one of 64 .. 1024 (Q = 1) or 1536, 2048 (Q = 2, nz <= 4), or a
+// plane above a CTA's shared memory.
+struct PassBG {
+  int H, M, Q;
+  int cols, pitch;      // columns per warp transform, complex values from column to column (one class)
+};
+bool passb_g_shape(const Grid& g, PassBG* s);
+// Whether pass B of this launch shape (engine without MMP_ENGINE_TC_Y) runs it.
+//   Block engine (0): R = 1.
+//   Warp engine (1): the classes R of the shape are the Q of the grid, except
+//   where one plane fills an SM (nz = 8 at Py = 1024, nz >= 4 at Py = 2048),
+//   which stays with the one-CTA-per-plane and two-CTA-cluster kernels of
+//   passb_w.cuh.
+bool passb_g_use(const Grid& g, int R, int warp_engine);
+// Planes per CTA, threads and dynamic shared memory; `nplanes` > 0: no more
+// planes per CTA than leave two CTAs per SM.
+struct PassBGLaunch { int kp, threads; size_t smem; };
+PassBGLaunch passb_g_plan(const Grid& g, const PassBG& s, int nplanes);
+struct BatchInst;
+struct BatchItem;
+// items null: the kx planes of g; else one CTA per work-list item.
+cudaError_t launch_passB_g(const Grid& g, const DemagArgs& d, const PassBG& s, const PassBGLaunch& l, int nblocks,
+                           const BatchInst* insts, const BatchItem* items, cudaStream_t st);
+
 // whether the tensor-core DFT32 stage applies on top of the warp pass B
 inline bool passb_tc_supported(const Grid& g, int R) { return passb_w_supported(g, R); }
 cudaError_t launch_field(const Grid& g, const DemagArgs& d, const Coefs& c, const FieldArgs& f,

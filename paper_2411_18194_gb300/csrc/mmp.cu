@@ -459,7 +459,10 @@ int apply_shape(mmp_ctx* ctx, const mmp_shape& s) {
   make_plan(g.Py / s.R, ctx->plan_ly, s.radix_y);
   TRY(upload_table(ctx, ctx->d_tw_x, pass_twiddles(ctx->plan_x)));
   TRY(upload_table(ctx, ctx->d_tw_ly, pass_twiddles(ctx->plan_ly)));
+  PassBG bg;
   if (s.engine & MMP_ENGINE_WARP_B) TRY(upload_table(ctx, ctx->d_tw_wy, warp_twiddles(g.Py / s.R)));
+  else if (passb_g_use(g, s.R, 0) && passb_g_shape(g, &bg))
+    TRY(upload_table(ctx, ctx->d_tw_wy, warp_twiddles(g.Py / bg.Q)));
   if ((s.engine & MMP_ENGINE_TC_Y) && !ctx->d_tw_tc) {
     const std::vector<float> t = tc_dft32_table();
     TRY(alloc_into(ctx, ctx->d_tw_tc, t.size() * sizeof(float)));

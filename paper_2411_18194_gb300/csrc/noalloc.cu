@@ -126,8 +126,11 @@ int set_up(Setup& S, int nx, int ny, int nz, const double* cell, cudaStream_t s)
     return cudaMemcpyAsync(b + off, src, bytes, cudaMemcpyHostToDevice, s);
   };
   cudaError_t e = cudaSuccess;
-  std::vector<float2> wx = pass_twiddles(d.plan_x), wy = roots(g.Py), wly = pass_twiddles(d.plan_ly),
-                     wz = roots(g.Pz);
+  // the general pass B takes its table in the place of the block engine's (of at least its length)
+  PassBG bg;
+  const bool gen = passb_g_use(g, R, 0) && passb_g_shape(g, &bg);
+  std::vector<float2> wx = pass_twiddles(d.plan_x), wy = roots(g.Py),
+                     wly = gen ? warp_twiddles(g.Py / bg.Q) : pass_twiddles(d.plan_ly), wz = roots(g.Pz);
   if (e == cudaSuccess) e = put(L.tw_x, wx.data(), wx.size() * sizeof(float2));
   if (e == cudaSuccess) e = put(L.tw_y, wy.data(), wy.size() * sizeof(float2));
   if (e == cudaSuccess) e = put(L.tw_ly, wly.data(), wly.size() * sizeof(float2));
@@ -170,6 +173,7 @@ int set_up(Setup& S, int nx, int ny, int nz, const double* cell, cudaStream_t s)
   d.tw_y = reinterpret_cast<const float2*>(b + L.tw_y);
   d.tw_ly = reinterpret_cast<const float2*>(b + L.tw_ly);
   d.tw_z = reinterpret_cast<const float2*>(b + L.tw_z);
+  d.tw_wy = d.tw_ly;
   d.R = R;
   S.g = g;
   S.d = d;

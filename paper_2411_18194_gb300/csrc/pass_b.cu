@@ -46,6 +46,11 @@ static cudaError_t launch_passB_t(const Grid& g, const DemagArgs& d, int threads
 }
 
 cudaError_t launch_passB(const Grid& g, const DemagArgs& d, int threads, cudaStream_t s) {
+  PassBG bg;
+  if (d.engine < 2 && passb_g_use(g, d.R, d.engine) && passb_g_shape(g, &bg)) {
+    const PassBGLaunch l = passb_g_plan(g, bg, g.kxn);
+    return launch_passB_g(g, d, bg, l, (g.kxn + l.kp - 1) / l.kp, nullptr, nullptr, s);
+  }
   if (d.engine == 1) {
     switch (g.Py / d.R) {
       case 256: return launch_passB_w_len<8>(g, d, s);
