@@ -22,7 +22,8 @@ OUT = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT, "libmmp.so")
 CHECKED_LIB = os.path.join(OUT, "checked", "libmmp_checked.so")
 SOURCES = ["mmp.cu", "pass_a.cu", "pass_b.cu", "field.cu", "elastic.cu", "tensor.cu", "noalloc.cu", "batch.cu", "batch_a.cu", "batch_b.cu", "batch_c.cu", "energy.cu", "passb_w8.cu", "passb_w16.cu", "passb_w32.cu", "passa_w.cu", "field_w.cu", "peak.cu", "batch_w.cu",
-           "passb_g.cu", "passb_g_a.cu", "passb_g_b.cu", "passb_g_c.cu", "passb_g_d.cu", "passb_g_e.cu"]
+           "passb_g.cu", "passb_g_a.cu", "passb_g_b.cu", "passb_g_c.cu", "passb_g_d.cu", "passb_g_e.cu",
+           "xfft_g.cu"] + ["xfft_g_%s.cu" % c for c in "ihgfedcba"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SPILL_LIMIT = 1024   # bytes of spill stores per thread
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"),

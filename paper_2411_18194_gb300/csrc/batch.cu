@@ -91,7 +91,7 @@ struct Launch {
   int off, cnt;
   size_t smem;
   int warp = -1;   // >= 0: the warp-engine launch of this pass for descriptor `warp`
-  bool general = false;   // pass B on the general warp kernel (passb_g.cuh), one CTA per item
+  bool general = false;   // on the general warp kernels (xfft_g.cuh, passb_g.cuh), one CTA per item
   PassBG bg{};
   PassBGLaunch bl{};
   Grid g{};        // its grid
@@ -223,10 +223,10 @@ BatchInst make_inst(const Member& m, unsigned* red, double h, int relax) {
   I.d.R = 1;
   I.d.ks = 0;
   I.d.tw_wy = c->d_tw_wy;
-  if (warp_member(c)) {   // the warp passes' tables and ky classes
+  I.d.tw_wx = c->d_tw_wx;
+  I.d.tw_wx2 = c->d_tw_wx2;
+  if (warp_member(c)) {   // the warp pass B's ky classes
     I.d.R = c->R;
-    I.d.tw_wx = c->d_tw_wx;
-    I.d.tw_wx2 = c->d_tw_wx2;
     I.d.err = c->d_flag;
     I.d.engine = 1;
   }
@@ -256,7 +256,7 @@ int build_list(mmp_batch* b, const std::vector<int>& mem) {
   L.members = mem;
   std::map<std::tuple<int, int, int>, std::vector<std::pair<double, BatchItem>>> sec;
   std::map<std::tuple<int, int, int>, size_t> smem;
-  std::map<std::tuple<int, int, int>, Launch> general;   // pass B sections of the general warp kernel
+  std::map<std::tuple<int, int, int>, Launch> general;   // sections of the general warp kernels
   std::vector<Launch> warp;   // the warp-engine members' launches
   for (int k = 0; k < (int)mem.size(); ++k) {
     const mmp_ctx* c = b->members[mem[k]].ctx;
@@ -291,10 +291,25 @@ int build_list(mmp_batch* b, const std::vector<int>& mem) {
     const auto ka = std::make_tuple(0, 0, thread_class(c->thrA));
     const auto kb = std::make_tuple(1, nz_group(g.nz), thread_class(c->thrB));
     const auto kc = std::make_tuple(2, 0, thread_class(c->thrC));
-    smem[ka] = std::max(smem[ka], smem_a(g));
     if (!gb) smem[kb] = std::max(smem[kb], smem_b(g));
-    smem[kc] = std::max(smem[kc], smem_c(g));
-    for (int z = 0; z < g.nz; ++z) {
+    // passes A and C on the general warp kernels: one launch per padded x
+    // length and block size, one item per row pair
+    int xm = 0, xq = 0;
+    const bool gx = xg_shape(g, &xm, &xq);
+    for (int kind = 0; gx && kind < 3; kind += 2) {
+      const auto key = std::make_tuple(kind, 1000 + g.Px, xg_plan(g, kind, (g.nx & 3) != 0).threads);
+      Launch& l = general[key];
+      l.general = true;
+      l.g = g;
+      for (int z = 0; z < g.nz; ++z)
+        for (int t = 0; t < (g.ny + 1) / 2; ++t)
+          sec[key].push_back({(double)(g.Px * (kind ? 2 : 1)), BatchItem{k, t, z}});
+    }
+    if (!gx) {
+      smem[ka] = std::max(smem[ka], smem_a(g));
+      smem[kc] = std::max(smem[kc], smem_c(g));
+    }
+    for (int z = 0; !gx && z < g.nz; ++z) {
       for (int t = 0; t < tiles; ++t) sec[ka].push_back({item_cost(g, 0), BatchItem{k, t, z}});
       for (int t = 0; t < tiles_c; ++t) sec[kc].push_back({item_cost(g, 2), BatchItem{k, t, z}});
     }
@@ -371,6 +386,7 @@ struct BTraced {
 cudaError_t launch_one(mmp_batch* b, const Launch& l, int stage, cudaStream_t s) {
   if (l.warp >= 0) return launch_batch_warp(l.kind, b->d_inst, l.warp, l.g, l.R, stage, s);
   const BatchItem* it = b->d_items + l.off;
+  if (l.general && l.kind != 1) return launch_xg_batch(l.kind, l.g, b->d_inst, it, l.cnt, stage, s);
   if (l.kind == 0) return launch_batch_passA(b->d_inst, it, l.cnt, stage, l.threads, l.smem, s);
   if (l.general) return launch_passB_g(l.g, DemagArgs{}, l.bg, l.bl, l.cnt, b->d_inst, it, s);
   if (l.kind == 1) return launch_batch_passB(l.group, b->d_inst, it, l.cnt, l.threads, l.smem, s);

@@ -24,6 +24,9 @@ size_t smem_field(const Grid& g, bool demag) {
 
 cudaError_t launch_field(const Grid& g, const DemagArgs& d, const Coefs& c, const FieldArgs& f, int nsub,
                          bool demag, int threads, cudaStream_t s) {
+  int M, Q;
+  if (demag && xg_shape(g, &M, &Q))
+    return launch_xg(2, (c.uniform ? 0 : 1) + (nsub == 2 ? 2 : 0), g, nullptr, d, c, &f, s);
   dim3 grid((g.ny + g.tyc - 1) / g.tyc, g.nz);
   size_t sm = smem_field(g, demag);
   cudaError_t e;

@@ -196,6 +196,41 @@ struct BatchItem;
 cudaError_t launch_passB_g(const Grid& g, const DemagArgs& d, const PassBG& s, const PassBGLaunch& l, int nblocks,
                            const BatchInst* insts, const BatchItem* items, cudaStream_t st);
 
+// General warp passes A and C (xfft_g.cuh): padded x lengths Px = Q * 32 M of
+// 64 .. 4096, one row pair per CTA.  Everything one tile needs:
+struct XgArgs {
+  Grid g;
+  DemagArgs d;
+  Coefs co;
+  StageArgs a;   // pass A
+  FieldArgs f;   // pass C
+};
+// Complex values from transform to transform: three components of a warp on
+// different banks, classes of kx too.
+__host__ __device__ constexpr int xg_pitch(int M, int Q) {
+  return (32 * M + (M < 16 ? M : Q > 1 ? 8 : 0) + 1) & ~1;
+}
+// Bytes of pass C's gathered spectrum, reused by its transforms.
+__host__ __device__ constexpr size_t xg_gather_bytes(int M, int Q) {
+  return (size_t)48 * (16 * M * Q + 1) > (size_t)24 * Q * xg_pitch(M, Q) ? (size_t)48 * (16 * M * Q + 1)
+                                                                          : (size_t)24 * Q * xg_pitch(M, Q);
+}
+__host__ __device__ constexpr int xg_maxthr(int Q) { return Q == 4 ? 384 : 256; }
+__host__ __device__ constexpr int xg_minblk(int Q) { return Q == 4 ? 1 : 2; }
+// M and Q of the grid; false outside the engine (Px < 64).
+bool xg_shape(const Grid& g, int* M, int* Q);
+// Threads and dynamic shared memory of pass 0 (A) or 2 (C); cells: pass C
+// works cell by cell.
+struct XgPlan { int threads; size_t smem; };
+XgPlan xg_plan(const Grid& g, int pass, bool cells);
+// One pass over the row pairs of g.  kind (pass C): bit 0 several regions, bit
+// 1 two sublattices.
+cudaError_t launch_xg(int pass, int kind, const Grid& g, const StageArgs* a, const DemagArgs& d, const Coefs& c,
+                      const FieldArgs* f, cudaStream_t st);
+// One pass over the items (member, row pair, z) of batch members of one Px.
+cudaError_t launch_xg_batch(int pass, const Grid& g, const BatchInst* insts, const BatchItem* items, int nitems,
+                            int stage, cudaStream_t st);
+
 // whether the tensor-core DFT32 stage applies on top of the warp pass B
 inline bool passb_tc_supported(const Grid& g, int R) { return passb_w_supported(g, R); }
 cudaError_t launch_field(const Grid& g, const DemagArgs& d, const Coefs& c, const FieldArgs& f,

@@ -468,11 +468,10 @@ int apply_shape(mmp_ctx* ctx, const mmp_shape& s) {
     TRY(alloc_into(ctx, ctx->d_tw_tc, t.size() * sizeof(float)));
     CK(cudaMemcpy(ctx->d_tw_tc, t.data(), t.size() * sizeof(float), cudaMemcpyHostToDevice), "upload tensor-core table");
   }
-  if (s.engine & MMP_ENGINE_WARP_X) {
-    TRY(upload_table(ctx, ctx->d_tw_wx, warp_twiddles(g.Px / 2)));
-    std::vector<float2> w = roots(g.Px);
-    w.resize(g.Px / 2);
-    TRY(upload_table(ctx, ctx->d_tw_wx2, w));
+  int xm = 0, xq = 0;   // passes A and C: the warp transforms of both engines (Px = 2048: the same tables)
+  if (xg_shape(g, &xm, &xq)) {
+    TRY(upload_table(ctx, ctx->d_tw_wx, warp_twiddles(g.Px / xq)));
+    TRY(upload_table(ctx, ctx->d_tw_wx2, roots(g.Px)));
   }
   g.ty = s.ty;
   g.tyc = s.tyc ? s.tyc : pick_tile_rows_c(s.ty, g.Px);

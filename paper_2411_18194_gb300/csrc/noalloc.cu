@@ -129,7 +129,12 @@ int set_up(Setup& S, int nx, int ny, int nz, const double* cell, cudaStream_t s)
   // the general pass B takes its table in the place of the block engine's (of at least its length)
   PassBG bg;
   const bool gen = passb_g_use(g, R, 0) && passb_g_shape(g, &bg);
-  std::vector<float2> wx = pass_twiddles(d.plan_x), wy = roots(g.Py),
+  // the general passes A and C: their transform table (one class) or the roots
+  // of Px (several) in the place of the block engine's; the transform table of
+  // several classes goes into the build's scratch afterwards
+  int xm = 0, xq = 0;
+  const bool xg = xg_shape(g, &xm, &xq);
+  std::vector<float2> wx = !xg ? pass_twiddles(d.plan_x) : xq == 1 ? warp_twiddles(g.Px) : roots(g.Px), wy = roots(g.Py),
                      wly = gen ? warp_twiddles(g.Py / bg.Q) : pass_twiddles(d.plan_ly), wz = roots(g.Pz);
   if (e == cudaSuccess) e = put(L.tw_x, wx.data(), wx.size() * sizeof(float2));
   if (e == cudaSuccess) e = put(L.tw_y, wy.data(), wy.size() * sizeof(float2));
@@ -165,6 +170,11 @@ int set_up(Setup& S, int nx, int ny, int nz, const double* cell, cudaStream_t s)
   kb.out = reinterpret_cast<float*>(b + L.khat);
   kb.krow = g.krow;
   e = build_kernel_spectrum(kb, s);
+  std::vector<float2> wcls;
+  if (xg && xq > 1) {
+    wcls = warp_twiddles(g.Px / xq);   // Px / xq <= 1.5 nx values in 48 nx ny nz bytes
+    if (e == cudaSuccess) e = put(L.buf0, wcls.data(), wcls.size() * sizeof(float2));
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_err(e, "mmp_demag_noalloc kernel build");
   d.T = reinterpret_cast<float2*>(b + L.T);
@@ -174,6 +184,8 @@ int set_up(Setup& S, int nx, int ny, int nz, const double* cell, cudaStream_t s)
   d.tw_ly = reinterpret_cast<const float2*>(b + L.tw_ly);
   d.tw_z = reinterpret_cast<const float2*>(b + L.tw_z);
   d.tw_wy = d.tw_ly;
+  d.tw_wx = xg && xq > 1 ? reinterpret_cast<const float2*>(b + L.buf0) : d.tw_x;
+  d.tw_wx2 = d.tw_x;
   d.R = R;
   S.g = g;
   S.d = d;

@@ -51,6 +51,8 @@ cudaError_t launch_normalize(float* m, long long n, cudaStream_t s) {
 
 cudaError_t launch_passA(const Grid& g, const StageArgs& a, const DemagArgs& d, const Coefs& c, int threads,
                          cudaStream_t s) {
+  int M, Q;
+  if (xg_shape(g, &M, &Q)) return launch_xg(0, 0, g, &a, d, c, nullptr, s);
   dim3 grid((g.ny + g.ty - 1) / g.ty, g.nz);
   size_t sm = smem_passA_launch(g, a);
   bool assemble = a.stage != nullptr && a.y != nullptr;

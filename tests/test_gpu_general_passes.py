@@ -51,3 +51,27 @@ def test_pass_b_lengths(ny, nz):
 def test_pass_b_default_shapes(ny, nz):
     """The creation defaults that run the general pass B under the warp engine."""
     check((6, ny, nz), 400 + ny, nreg=2, empty=0.05)
+
+
+# passes A and C (xfft_g.cuh): padded x lengths 64 .. 1024 (one class of kx), 1536 and 2048 (two), 3072 and
+# 4096 (four): smallest and largest nx of each, odd ones and ones of 2 mod 4 among them, ny odd, even and 1
+ROWS = [(25, 4, 2), (32, 5, 1), (33, 6, 1), (48, 1, 3), (49, 7, 1), (64, 8, 2), (66, 3, 2), (96, 4, 1), (97, 2, 1),
+        (128, 5, 3), (130, 6, 1), (192, 3, 1), (193, 4, 1), (256, 9, 2), (258, 2, 1), (384, 4, 1), (387, 3, 2),
+        (512, 6, 1), (514, 5, 1), (768, 4, 2), (771, 2, 1), (1024, 3, 1), (1025, 4, 1), (1536, 2, 1), (1538, 3, 1),
+        (2047, 2, 1), (2048, 5, 1)]
+
+
+@pytest.mark.parametrize("nx,ny,nz", ROWS)
+def test_passes_a_and_c_lengths(nx, ny, nz):
+    from paper_2411_18194_gb300 import MmpError
+    try:   # engine 0: the general passes at Px = 2048 too
+        check((nx, ny, nz), 500 + nx + ny, R=1, stage_kernel=0, engine=0)
+    except MmpError:
+        check((nx, ny, nz), 500 + nx + ny)
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(31, 6, 2), (100, 7, 1), (300, 4, 2), (700, 3, 1), (1030, 4, 1), (2000, 2, 1)])
+def test_passes_a_and_c_materials(nx, ny, nz):
+    """Several regions with empty cells, and two sublattices."""
+    check((nx, ny, nz), 600 + nx, nreg=3, empty=0.1)
+    check((nx, ny, nz), 700 + nx, n_sub=2, terms=("DEMAG", "EXCH", "ANIS", "AFM", "ZEEMAN"))
