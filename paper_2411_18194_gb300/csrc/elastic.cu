@@ -75,27 +75,48 @@ __device__ __forceinline__ bool in_bulk(const int (&idx)[3], const int (&ext)[3]
   return b;
 }
 
-__global__ void k_strain(Grid g, ElasticArgs e, int nsub) {
+// Cells of row z ny + y by x: one thread a cell, rows over blockIdx.y (no
+// division by the extents).
+constexpr int kElThreads = 128;
+static dim3 elastic_grid(const Grid& g) {
+  const long long rows = (long long)g.ny * g.nz;
+  return dim3((g.nx + kElThreads - 1) / kElThreads, (unsigned)(rows < 65535 ? rows : 65535));
+}
+
+// Both elastic kernels are bound by the latency of their neighbour loads (24 and
+// about 80 a cell): a cell whose rows are all in the 4th-order bulk takes a path
+// with no selection between them, so that they are in flight together; the
+// selection per term and the 64-bit divisions of the index took most of the time
+// before: 25 and 59 us per launch at 1024x256x1 with two sublattices (cold L2).
+// Antiferromagnet 1024x256x1, four steps (25 launches of each): 4506 -> 3994 us.
+// HZ: nz > 1.
+template <bool HZ>
+__global__ void __launch_bounds__(kElThreads) k_strain(Grid g, ElasticArgs e, int nsub) {
   const long long n = g.n;
   const float* u = e.stage + (long long)3 * nsub * n;
   const float* v = u + 3 * n;
-  for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < n;
-       cell += (long long)gridDim.x * blockDim.x) {
-    int x = cell % g.nx, y = (cell / g.nx) % g.ny, z = cell / ((long long)g.nx * g.ny);
+  const int x = blockIdx.x * kElThreads + threadIdx.x;
+  if (x >= g.nx) return;
+  constexpr int NA = HZ ? 3 : 2;
+  for (int row = blockIdx.y; row < g.ny * g.nz; row += gridDim.y) {
+    const int z = HZ ? row / g.ny : 0, y = row - z * g.ny;
+    const long long cell = x + (long long)g.nx * row;
     const int idx[3] = {x, y, z}, ext[3] = {g.nx, g.ny, g.nz};
     const long long st[3] = {1, g.nx, (long long)g.nx * g.ny};
-    float G[3][3], Gv[3][3];
+    float G[3][3] = {}, Gv[3][3] = {};
     if (in_bulk(idx, ext, 2)) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+      for (int a = 0; a < NA; ++a)
+        if (ext[a] > 1) {
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          G[a][j] = ext[a] > 1 ? grad_bulk(u + j * n, cell, st[a], g.ih[a]) : 0.0f;
-          Gv[a][j] = e.eta != 0.0f && ext[a] > 1 ? grad_bulk(v + j * n, cell, st[a], g.ih[a]) : 0.0f;
+          for (int j = 0; j < 3; ++j) G[a][j] = grad_bulk(u + j * n, cell, st[a], g.ih[a]);
+          if (e.eta != 0.0f)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) Gv[a][j] = grad_bulk(v + j * n, cell, st[a], g.ih[a]);
         }
     } else {
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+      for (int a = 0; a < NA; ++a)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
           G[a][j] = grad_at(u + j * n, cell, idx[a], ext[a], st[a], g.ih[a]);
@@ -128,63 +149,82 @@ __global__ void k_strain(Grid g, ElasticArgs e, int nsub) {
   }
 }
 
-template <bool UNI>
-__global__ void k_elastic_rhs(Grid g, ElasticArgs e, Coefs co, int nsub) {
+// Force of one cell.  BULK: every row of G and G^T it needs is in the bulk.
+template <bool UNI, bool HZ, bool BULK>
+__device__ __forceinline__ void elastic_force(const Grid& g, const ElasticArgs& e, const Coefs& co, int nsub,
+                                              long long cell, const int (&idx)[3], float (&f)[3]) {
   const long long n = g.n;
-  const float* u = e.stage + (long long)3 * nsub * n;
-  const float* v = u + 3 * n;
+  constexpr int NA = HZ ? 3 : 2;
+  constexpr int sidx[3][3] = {{0, 3, 4}, {3, 1, 5}, {4, 5, 2}};   // sigma_ab as component of sig[6]
+  const int ext[3] = {g.nx, g.ny, g.nz};
+  const long long st[3] = {1, g.nx, (long long)g.nx * g.ny};
+#pragma unroll
+  for (int a = 0; a < NA; ++a)
+    if (!BULK || ext[a] > 1)
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+        f[b] -= BULK ? gradT_bulk(e.sig + sidx[a][b] * n, cell, st[a], g.ih[a])
+                     : gradT_at(e.sig + sidx[a][b] * n, cell, idx[a], ext[a], st[a], g.ih[a]);
+  if (!(e.terms & 64u)) return;
+  const int reg = UNI ? 0 : co.regions[cell];
+  for (int s = 0; s < nsub; ++s) {
+    const float* m = e.stage + (long long)3 * s * n;
+    const RegionCoef& R = co.reg[s * MMP_MAX_REGIONS + reg];
+    float G[3][3] = {};
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+      if (!BULK || ext[a] > 1)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          G[a][j] = BULK ? grad_bulk(m + j * n, cell, st[a], g.ih[a])
+                         : grad_at(m + j * n, cell, idx[a], ext[a], st[a], g.ih[a]);
+    const float mx = m[cell], my = m[n + cell], mz = m[2 * n + cell];
+    const float B1 = R.b1, B2 = R.b2;
+    f[0] += 2.0f * B1 * mx * G[0][0] + B2 * (mx * (G[1][1] + G[2][2]) + my * G[1][0] + mz * G[2][0]);
+    f[1] += 2.0f * B1 * my * G[1][1] + B2 * (my * (G[0][0] + G[2][2]) + mx * G[0][1] + mz * G[2][1]);
+    f[2] += 2.0f * B1 * mz * G[2][2] + B2 * (mz * (G[0][0] + G[1][1]) + mx * G[0][2] + my * G[1][2]);
+  }
+}
+
+template <bool UNI, bool HZ>
+__global__ void __launch_bounds__(kElThreads) k_elastic_rhs(Grid g, ElasticArgs e, Coefs co, int nsub) {
+  const long long n = g.n;
+  const float* v = e.stage + (long long)3 * (nsub + 1) * n;
   float* ku = e.kout + (long long)3 * nsub * n;
   float* kv = ku + 3 * n;
-  // sigma_ab as component index into sig[6]
-  const int sidx[3][3] = {{0, 3, 4}, {3, 1, 5}, {4, 5, 2}};
-  for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < n;
-       cell += (long long)gridDim.x * blockDim.x) {
-    int x = cell % g.nx, y = (cell / g.nx) % g.ny, z = cell / ((long long)g.nx * g.ny);
+  const int x = blockIdx.x * kElThreads + threadIdx.x;
+  if (x >= g.nx) return;
+  for (int row = blockIdx.y; row < g.ny * g.nz; row += gridDim.y) {
+    const int z = HZ ? row / g.ny : 0, y = row - z * g.ny;
+    const long long cell = x + (long long)g.nx * row;
     const int idx[3] = {x, y, z}, ext[3] = {g.nx, g.ny, g.nz};
-    const long long st[3] = {1, g.nx, (long long)g.nx * g.ny};
+    const float vc[3] = {v[cell], v[n + cell], v[2 * n + cell]};
     float f[3] = {0.0f, 0.0f, 0.0f};
-    const bool bulkT = in_bulk(idx, ext, 4), bulk = in_bulk(idx, ext, 2);
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-        f[b] -= bulkT ? (ext[a] > 1 ? gradT_bulk(e.sig + sidx[a][b] * n, cell, st[a], g.ih[a]) : 0.0f)
-                      : gradT_at(e.sig + sidx[a][b] * n, cell, idx[a], ext[a], st[a], g.ih[a]);
-    if (e.terms & 64u) {
-      int reg = UNI ? 0 : co.regions[cell];
-      for (int s = 0; s < nsub; ++s) {
-        const float* m = e.stage + (long long)3 * s * n;
-        const RegionCoef& R = co.reg[s * MMP_MAX_REGIONS + reg];
-        float G[3][3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-          for (int j = 0; j < 3; ++j)
-            G[a][j] = bulk ? (ext[a] > 1 ? grad_bulk(m + j * n, cell, st[a], g.ih[a]) : 0.0f)
-                           : grad_at(m + j * n, cell, idx[a], ext[a], st[a], g.ih[a]);
-        float mx = m[cell], my = m[n + cell], mz = m[2 * n + cell];
-        float B1 = R.b1, B2 = R.b2;
-        f[0] += 2.0f * B1 * mx * G[0][0] + B2 * (mx * (G[1][1] + G[2][2]) + my * G[1][0] + mz * G[2][0]);
-        f[1] += 2.0f * B1 * my * G[1][1] + B2 * (my * (G[0][0] + G[2][2]) + mx * G[0][1] + mz * G[2][1]);
-        f[2] += 2.0f * B1 * mz * G[2][2] + B2 * (mz * (G[0][0] + G[1][1]) + mx * G[0][2] + my * G[1][2]);
-      }
-    }
+    if (in_bulk(idx, ext, 4)) elastic_force<UNI, HZ, true>(g, e, co, nsub, cell, idx, f);
+    else elastic_force<UNI, HZ, false>(g, e, co, nsub, cell, idx, f);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      ku[c * n + cell] = v[c * n + cell];
+      ku[c * n + cell] = vc[c];
       kv[c * n + cell] = f[c] * e.inv_rho;
     }
   }
 }
 
 cudaError_t launch_strain(const Grid& g, const ElasticArgs& e, int nsub, cudaStream_t s) {
-  k_strain<<<grid_for(g.n, 256), 256, 0, s>>>(g, e, nsub);
+  if (g.nz > 1) k_strain<true><<<elastic_grid(g), kElThreads, 0, s>>>(g, e, nsub);
+  else k_strain<false><<<elastic_grid(g), kElThreads, 0, s>>>(g, e, nsub);
   return cudaGetLastError();
 }
 
 cudaError_t launch_elastic_rhs(const Grid& g, const ElasticArgs& e, const Coefs& c, int nsub, cudaStream_t s) {
-  if (c.uniform) k_elastic_rhs<true><<<grid_for(g.n, 256), 256, 0, s>>>(g, e, c, nsub);
-  else k_elastic_rhs<false><<<grid_for(g.n, 256), 256, 0, s>>>(g, e, c, nsub);
+  const dim3 grid = elastic_grid(g);
+  if (c.uniform) {
+    if (g.nz > 1) k_elastic_rhs<true, true><<<grid, kElThreads, 0, s>>>(g, e, c, nsub);
+    else k_elastic_rhs<true, false><<<grid, kElThreads, 0, s>>>(g, e, c, nsub);
+  } else {
+    if (g.nz > 1) k_elastic_rhs<false, true><<<grid, kElThreads, 0, s>>>(g, e, c, nsub);
+    else k_elastic_rhs<false, false><<<grid, kElThreads, 0, s>>>(g, e, c, nsub);
+  }
   return cudaGetLastError();
 }
 
