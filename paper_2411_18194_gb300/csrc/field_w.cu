@@ -14,12 +14,11 @@ cudaError_t launch_field_w(const Grid& g, const DemagArgs& d, const Coefs& c, co
 #define MMP_FW(NS, UN)                                                 \
   do {                                                                 \
     if ((e = set_smem(k_field_w<NS, UN>, sm)) != cudaSuccess) return e; \
-    k_field_w<NS, UN><<<grid, kXwThreads, sm, s>>>(g, d, c, f);         \
+    return launch_chained(d.chain, k_field_w<NS, UN>, grid, kXwThreads, sm, s, g, d, c, f); \
   } while (0)
   if (nsub == 1) { if (c.uniform) MMP_FW(1, true); else MMP_FW(1, false); }
   else { if (c.uniform) MMP_FW(2, true); else MMP_FW(2, false); }
 #undef MMP_FW
-  return cudaGetLastError();
 }
 
 }  // namespace mmp

@@ -89,6 +89,7 @@ struct DemagArgs {
   const float2* tw_wx2;      // w_Px^x, x < Px / 2 (natural order; passes A and C)
   const float* tw_tc;        // tensor-core DFT32 matrices, split TF32 (tcdft.cuh layout)
   unsigned* err;             // set to 1 by a device wait that ran past its limit
+  int chain;                 // launch_chained for the warp passes (0 in captured graphs, see launch.cuh)
   int engine;                // pass B: 0 block engine, 1 warp passes, 2 warp passes with the final
                              // DFT32 of each y transform on the tensor cores; 0 and 1 run the
                              // general warp pass B where passb_g_use says so

@@ -524,6 +524,7 @@ DemagArgs demag_args(mmp_ctx* ctx) {
   d.tw_wx2 = ctx->d_tw_wx2;
   d.tw_tc = ctx->d_tw_tc;
   d.err = ctx->d_flag;
+  d.chain = !ctx->gstream || ctx->stream != ctx->gstream;   // gstream: captured into the fixed-step graph
   d.engine = (ctx->engine & MMP_ENGINE_WARP_B) ? ((ctx->engine & MMP_ENGINE_TC_Y) ? 2 : 1) : 0;
   return d;
 }

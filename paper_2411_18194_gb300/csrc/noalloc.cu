@@ -187,6 +187,7 @@ int set_up(Setup& S, int nx, int ny, int nz, const double* cell, cudaStream_t s)
   d.tw_wx = xg && xq > 1 ? reinterpret_cast<const float2*>(b + L.buf0) : d.tw_x;
   d.tw_wx2 = d.tw_x;
   d.R = R;
+  d.chain = 1;
   S.g = g;
   S.d = d;
   S.co.reg = reinterpret_cast<const RegionCoef*>(b + L.coef);

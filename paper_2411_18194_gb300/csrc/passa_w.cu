@@ -14,12 +14,11 @@ cudaError_t launch_passA_w(const Grid& g, const StageArgs& a, const DemagArgs& d
 #define MMP_PAW(NS, AS)                                                \
   do {                                                                 \
     if ((e = set_smem(k_passA_w<NS, AS>, sm)) != cudaSuccess) return e; \
-    k_passA_w<NS, AS><<<grid, kXwThreads, sm, s>>>(g, a, d, c);         \
+    return launch_chained(d.chain, k_passA_w<NS, AS>, grid, kXwThreads, sm, s, g, a, d, c); \
   } while (0)
   if (a.nsub == 1) { if (assemble) MMP_PAW(1, true); else MMP_PAW(1, false); }
   else { if (assemble) MMP_PAW(2, true); else MMP_PAW(2, false); }
 #undef MMP_PAW
-  return cudaGetLastError();
 }
 
 }  // namespace mmp

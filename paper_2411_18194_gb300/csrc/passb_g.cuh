@@ -29,6 +29,7 @@
 #include "batch.h"
 #include "kernels.h"
 #include "gfft.cuh"
+#include "launch.cuh"
 #include "passb_w.cuh"
 
 namespace mmp {
@@ -226,6 +227,7 @@ __global__ void __launch_bounds__(passb_g_maxthr(H), passb_g_minblk(H))
     k_passB_g(Grid g, DemagArgs d, int kp, const BatchInst* __restrict__ insts, const BatchItem* __restrict__ items) {
   extern __shared__ __align__(16) unsigned char sraw[];
   if (!insts) {
+    after_predecessor();
     const int kx0 = blockIdx.x * kp;
     passB_g_planes<H, M, Q>(sraw, g, d, kx0, min(kp, g.kxn - kx0));
   } else {
@@ -247,8 +249,9 @@ cudaError_t launch_passB_g_t(const Grid& g, const DemagArgs& d, const PassBGLaun
 template <int H, int M, int Q>
 cudaError_t launch_passB_g_t(const Grid& g, const DemagArgs& d, const PassBGLaunch& l, int nblocks,
                              const BatchInst* insts, const BatchItem* items, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(k_passB_g<H, M, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+  cudaError_t e = set_smem(k_passB_g<H, M, Q>, l.smem);
   if (e != cudaSuccess) return e;
+  if (!insts) return launch_chained(d.chain, k_passB_g<H, M, Q>, dim3(nblocks), l.threads, l.smem, st, g, d, l.kp, insts, items);
   k_passB_g<H, M, Q><<<nblocks, l.threads, l.smem, st>>>(g, d, l.kp, insts, items);
   return cudaGetLastError();
 }

@@ -25,6 +25,7 @@
 #include "field.cuh"
 #include "gfft.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 #include "stencil4.cuh"
 
 namespace mmp {
@@ -377,6 +378,7 @@ __device__ __forceinline__ BatchItem xg_tile(XgArgs& s, const XgArgs& p, const B
                                              const BatchItem* items, int stage) {
   if (!insts) {
     xg_copy(s, p);
+    after_predecessor();
     __syncthreads();
     return BatchItem{0, (int)blockIdx.x, (int)blockIdx.y};
   }
@@ -426,6 +428,7 @@ static cudaError_t xg_go(K kernel, const XgArgs& p, const XgLaunch& l, const Bat
                          int stage, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
   if (e != cudaSuccess) return e;
+  if (!insts) return launch_chained(p.d.chain, kernel, l.grid, l.threads, l.smem, st, p, insts, items, stage);
   kernel<<<l.grid, l.threads, l.smem, st>>>(p, insts, items, stage);
   return cudaGetLastError();
 }

@@ -21,6 +21,7 @@
 // per thread (field_cells) for two sublattices or several regions.
 #pragma once
 #include "kernels.h"
+#include "launch.cuh"
 #include "wfft.cuh"
 #include "copy.cuh"
 #include "stage.cuh"
@@ -423,12 +424,14 @@ __device__ __forceinline__ void field_w_tile(unsigned char* sraw, const Grid& g,
 template <int NSUB, bool ASSEMBLE>
 __global__ void __launch_bounds__(kXwThreads, 4) k_passA_w(Grid g, StageArgs a, DemagArgs d, Coefs co) {
   extern __shared__ __align__(16) unsigned char sraw[];
+  after_predecessor();
   passA_w_tile<NSUB, ASSEMBLE>(sraw, g, a, d, co, blockIdx.y, 2 * blockIdx.x);
 }
 
 template <int NSUB, bool UNI>
 __global__ void __launch_bounds__(kXwThreads, 4) k_field_w(Grid g, DemagArgs d, Coefs co, FieldArgs f) {
   extern __shared__ __align__(16) unsigned char sraw[];
+  after_predecessor();
   field_w_tile<NSUB, UNI>(sraw, g, d, co, f, blockIdx.y, 2 * blockIdx.x);
 }
 
