@@ -297,7 +297,7 @@ int build_list(mmp_batch* b, const std::vector<int>& mem) {
     int xm = 0, xq = 0;
     const bool gx = xg_shape(g, &xm, &xq);
     for (int kind = 0; gx && kind < 3; kind += 2) {
-      const auto key = std::make_tuple(kind, 1000 + g.Px, xg_plan(g, kind, (g.nx & 3) != 0).threads);
+      const auto key = std::make_tuple(kind, 1000 + g.Px, xg_plan(g, kind, (g.nx & 3) != 0, true).threads);
       Launch& l = general[key];
       l.general = true;
       l.g = g;

@@ -246,47 +246,38 @@ __device__ __forceinline__ void inverse_x_components(int c0, int nc, float2* fbu
   __syncthreads();
 }
 
-// Local field, torque and the reductions of rows y0 .. y0 + nrows - 1 of
-// plane z (one tile): bd is the demag field of the tile, component c, row
-// `row`, cell x at bd[c * cstride + row * rstride + x].
-template <int NSUB, bool DEMAG, bool UNI>
-__device__ __forceinline__ void field_cells(const float* bd, int cstride, int rstride, int nrows, const Grid& g,
-                                            const Coefs& co, const FieldArgs& f, int z, int y0) {
-  const int nx = g.nx, ny = g.ny;
-  float emax = 0.0f, tmax = 0.0f;
+// Local field and torque of one cell of demag field b3, with its error estimate
+// and torque maximum (both NaN-keeping).
+template <int NSUB, bool UNI>
+__device__ __forceinline__ void field_cell(const float* b3, const Grid& g, const Coefs& co, const FieldArgs& f, int x,
+                                           int y, int z, long long cell, float& emax, float& tmax) {
+  if (!MMP_IN(g, cell, g.n)) return;
   const long long n = g.n;
-  for (int e = threadIdx.x; e < nrows * nx; e += blockDim.x) {
-    int row = e / nx, x = e - row * nx, y = y0 + row;
-    if (y >= ny) continue;
-    long long cell = x + (long long)nx * (y + (long long)ny * z);
-    if (!MMP_IN(g, cell, g.n)) continue;
-    int reg = UNI ? 0 : co.regions[cell];
-    float b3[3] = {0.0f, 0.0f, 0.0f};
-    if (DEMAG) {
+  const int reg = UNI ? 0 : co.regions[cell];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) b3[c] = bd[c * cstride + row * rstride + x];
-    }
+  for (int s = 0; s < NSUB; ++s) {
+    CellOut o = cell_field<UNI, NSUB>(g, co, f, s, x, y, z, cell, reg, b3);
 #pragma unroll
-    for (int s = 0; s < NSUB; ++s) {
-      CellOut o = cell_field<UNI, NSUB>(g, co, f, s, x, y, z, cell, reg, b3);
+    for (int i = 0; i < 3; ++i) {
+      long long idx = (long long)(3 * s + i) * n + cell;
+      if (!MMP_IN(g, idx, g.lim_B)) continue;
+      f.kout[idx] = o.tau[i];
+      if (f.Bout) f.Bout[idx] = o.B[i];
+      if (f.err) {
+        float ev = f.ecoef[6] * o.tau[i];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        long long idx = (long long)(3 * s + i) * n + cell;
-        if (!MMP_IN(g, idx, g.lim_B)) continue;
-        f.kout[idx] = o.tau[i];
-        if (f.Bout) f.Bout[idx] = o.B[i];
-        if (f.err) {
-          float ev = f.ecoef[6] * o.tau[i];
-#pragma unroll
-          for (int j = 0; j < 6; ++j)
-            if (f.ecoef[j] != 0.0f) ev = fmaf(f.ecoef[j], f.ek[j][idx], ev);
-          ev = fabsf(ev);
-          emax = isnan(ev) || ev > emax ? ev : emax;
-        }
+        for (int j = 0; j < 6; ++j)
+          if (f.ecoef[j] != 0.0f) ev = fmaf(f.ecoef[j], f.ek[j][idx], ev);
+        ev = fabsf(ev);
+        emax = isnan(ev) || ev > emax ? ev : emax;
       }
-      tmax = isnan(o.mxb) || o.mxb > tmax ? o.mxb : tmax;
     }
+    tmax = isnan(o.mxb) || o.mxb > tmax ? o.mxb : tmax;
   }
+}
+
+// The block's error estimate and torque maximum into the launch's.
+__device__ __forceinline__ void field_maxima(const FieldArgs& f, float emax, float tmax) {
   if (f.err) {
     float v = block_max(isnan(emax) ? __int_as_float(0x7f800000) : emax);
     if (threadIdx.x == 0) atomic_max_pos(f.err, v);
@@ -295,6 +286,28 @@ __device__ __forceinline__ void field_cells(const float* bd, int cstride, int rs
     float v = block_max(isnan(tmax) ? __int_as_float(0x7f800000) : tmax);
     if (threadIdx.x == 0) atomic_max_pos(f.torque_max, v);
   }
+}
+
+// Local field, torque and the reductions of rows y0 .. y0 + nrows - 1 of
+// plane z (one tile): bd is the demag field of the tile, component c, row
+// `row`, cell x at bd[c * cstride + row * rstride + x].
+template <int NSUB, bool DEMAG, bool UNI>
+__device__ __forceinline__ void field_cells(const float* bd, int cstride, int rstride, int nrows, const Grid& g,
+                                            const Coefs& co, const FieldArgs& f, int z, int y0) {
+  const int nx = g.nx, ny = g.ny;
+  float emax = 0.0f, tmax = 0.0f;
+  for (int e = threadIdx.x; e < nrows * nx; e += blockDim.x) {
+    int row = e / nx, x = e - row * nx, y = y0 + row;
+    if (y >= ny) continue;
+    long long cell = x + (long long)nx * (y + (long long)ny * z);
+    float b3[3] = {0.0f, 0.0f, 0.0f};
+    if (DEMAG) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) b3[c] = bd[c * cstride + row * rstride + x];
+    }
+    field_cell<NSUB, UNI>(b3, g, co, f, x, y, z, cell, emax, tmax);
+  }
+  field_maxima(f, emax, tmax);
 }
 
 // Pass C of one tile: rows y0 .. y0 + ty - 1 of plane z.  `smem` is the

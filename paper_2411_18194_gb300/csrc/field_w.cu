@@ -8,17 +8,12 @@ namespace mmp {
 
 cudaError_t launch_field_w(const Grid& g, const DemagArgs& d, const Coefs& c, const FieldArgs& f, int nsub,
                            cudaStream_t s) {
+  const int kind = (c.uniform ? 0 : 1) + (nsub == 2 ? 2 : 0);
+  if (xg_split(g, kind)) return launch_xg(2, kind, g, nullptr, d, c, &f, s);   // every kind but 0
   const dim3 grid((g.ny + 1) / 2, g.nz);
   const size_t sm = field_w_smem();
-  cudaError_t e;
-#define MMP_FW(NS, UN)                                                 \
-  do {                                                                 \
-    if ((e = set_smem(k_field_w<NS, UN>, sm)) != cudaSuccess) return e; \
-    return launch_chained(d.chain, k_field_w<NS, UN>, grid, kXwThreads, sm, s, g, d, c, f); \
-  } while (0)
-  if (nsub == 1) { if (c.uniform) MMP_FW(1, true); else MMP_FW(1, false); }
-  else { if (c.uniform) MMP_FW(2, true); else MMP_FW(2, false); }
-#undef MMP_FW
+  const cudaError_t e = set_smem(k_field_w<1, true>, sm, 1024);
+  return e != cudaSuccess ? e : launch_chained(d.chain, k_field_w<1, true>, grid, kXwThreads, sm, s, g, d, c, f);
 }
 
 }  // namespace mmp

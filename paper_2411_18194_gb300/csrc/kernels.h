@@ -223,7 +223,9 @@ bool xg_shape(const Grid& g, int* M, int* Q);
 // Threads and dynamic shared memory of pass 0 (A) or 2 (C); cells: pass C
 // works cell by cell.
 struct XgPlan { int threads; size_t smem; };
-XgPlan xg_plan(const Grid& g, int pass, bool cells);
+XgPlan xg_plan(const Grid& g, int pass, bool cells, bool batch);
+// Whether pass C is two kernels for this grid and kind.
+bool xg_split(const Grid& g, int kind);
 // One pass over the row pairs of g.  kind (pass C): bit 0 several regions, bit
 // 1 two sublattices.
 cudaError_t launch_xg(int pass, int kind, const Grid& g, const StageArgs* a, const DemagArgs& d, const Coefs& c,

@@ -283,14 +283,7 @@ __device__ __forceinline__ void field_cells4(const float* msm, const float* bd, 
     const long long cell0 = x0 + (long long)nx * (y + (long long)g.ny * z);
     st4_item<DEMAG>(msm, bd, cs, rs, h, x0, nrows == 2, g, sR, f, z, y, cell0, emax, tmax);
   }
-  if (f.err) {
-    float v = block_max(isnan(emax) ? __int_as_float(0x7f800000) : emax);
-    if (threadIdx.x == 0) atomic_max_pos(f.err, v);
-  }
-  if (f.torque_max) {
-    float v = block_max(isnan(tmax) ? __int_as_float(0x7f800000) : tmax);
-    if (threadIdx.x == 0) atomic_max_pos(f.torque_max, v);
-  }
+  field_maxima(f, emax, tmax);
 }
 
 }  // namespace mmp

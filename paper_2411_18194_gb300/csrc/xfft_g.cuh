@@ -118,16 +118,17 @@ __device__ __forceinline__ void xg_store(const Grid& g, float* p, long long idx,
   else p[idx] = v.v[0];
 }
 
-// Assembly of both rows: items of V cells in each row; M into Z[c][x] = (row a, row b).
+// Assembly of both rows of the parts p0 .. p1 - 1: items of V cells in each row;
+// M of the sublattices into Z[c][x] = (row a, row b).
 template <int V>
 __device__ __forceinline__ void xg_assemble(const Grid& g, const StageArgs& a, const Coefs& co, float2* Z, int hx,
-                                            int z, int y0) {
+                                            int p0, int p1, int z, int y0) {
   const int nx = g.nx;
   const long long n = g.n, row0 = (long long)nx * (y0 + (long long)g.ny * z);
   const bool two = y0 + 1 < g.ny, assemble = a.y != nullptr, uni = co.uniform != 0;
-  const int nsub = a.nsub, nparts = a.nparts;
+  const int nsub = a.nsub;
   for (int x0 = V * threadIdx.x; x0 < nx; x0 += V * blockDim.x) {
-    for (int p = 0; p < (assemble ? nparts : nsub); ++p) {
+    for (int p = p0; p < p1; ++p) {
       const long long idx0 = 3LL * p * n + row0 + x0;
       VecF<V> v[3][2];
       xg_stage<V>(g, a, assemble, idx0, two, v);
@@ -172,8 +173,10 @@ __device__ __forceinline__ void xg_assemble(const Grid& g, const StageArgs& a, c
   }
 }
 
+// part 0: the sublattices and the transforms; part q > 0: elastic part q - 1,
+// assembled and not transformed, in a block of its own.
 template <int M, int Q>
-__device__ __forceinline__ void passA_g_tile(unsigned char* sraw, const XgArgs& s, int z, int y0) {
+__device__ __forceinline__ void passA_g_tile(unsigned char* sraw, const XgArgs& s, int part, int z, int y0) {
   using X = Xg<M, Q>;
   constexpr int NB = X::NB, N = X::N, LP = X::LP, HX = X::HX;
   constexpr bool HALF = Q == 1;
@@ -188,8 +191,10 @@ __device__ __forceinline__ void passA_g_tile(unsigned char* sraw, const XgArgs& 
   unsigned long long alk = 0;
 #pragma unroll
   for (int j = 0; j < 7; ++j) alk |= j < s.a.nk ? reinterpret_cast<unsigned long long>(s.a.k[j]) : 0ull;
-  if (!(nx & 1) && !((al | alk) & 7)) xg_assemble<2>(g, s.a, s.co, Z, HX, z, y0);
-  else xg_assemble<1>(g, s.a, s.co, Z, HX, z, y0);
+  const int p0 = part ? s.a.nsub + part - 1 : 0, p1 = part ? p0 + 1 : s.a.nsub;
+  if (!(nx & 1) && !((al | alk) & 7)) xg_assemble<2>(g, s.a, s.co, Z, HX, p0, p1, z, y0);
+  else xg_assemble<1>(g, s.a, s.co, Z, HX, p0, p1, z, y0);
+  if (part) return;
   __syncthreads();
   if (warp < X::GRP) {
     const int c0 = NB == 3 ? 0 : warp / Q, r = NB == 3 ? 0 : warp - c0 * Q;
@@ -387,7 +392,38 @@ __device__ __forceinline__ BatchItem xg_tile(XgArgs& s, const XgArgs& p, const B
   xg_copy(s.g, I.g);
   xg_copy(s.d, I.d);
   xg_copy(s.co, I.co);
-  if (threadIdx.x == 0) batch_args(I, stage, s.a, s.f);
+  // as batch_args, one entry a lane: by one thread this chain of loads from the
+  // descriptor lasted longer than a small tile's transforms
+  if (threadIdx.x < 32) {
+    const int j = threadIdx.x, p = I.par;
+    float* const k1 = I.kbuf[p];
+    float* const k7 = I.kbuf[p ^ 1];
+    float* kj = j == 0 ? k1 : j < 6 ? I.kmid[j - 1] : k7;
+    const bool last = stage == 6;
+    if (j < 7) {
+      s.a.k[j] = j < stage ? kj : nullptr;
+      s.a.coef[j] = j < stage ? I.coef[stage][j] : 0.0f;
+      s.f.ecoef[j] = last ? I.ecoef[j] : 0.0f;
+      if (j < 6) s.f.ek[j] = last ? kj : nullptr;
+      if (j == stage) s.f.kout = kj;
+    } else if (j == 7) {
+      float* st = I.ybuf[stage == 0 ? p : p ^ 1];
+      s.a.y = stage == 0 ? nullptr : I.ybuf[p];
+      s.a.stage = st;
+      s.f.stage = st;
+    } else if (j == 8) {
+      s.a.nk = stage;
+      s.a.normalize = last;
+      s.a.nparts = 1;
+      s.a.nsub = 1;
+      s.f.Bout = nullptr;
+      s.f.eps = nullptr;
+      s.f.terms = I.terms;
+      s.f.relax = I.relax;
+      s.f.err = last ? I.red : nullptr;
+      s.f.torque_max = last ? I.red + 1 : nullptr;
+    }
+  }
   __syncthreads();
   return w;
 }
@@ -399,7 +435,88 @@ __global__ void __launch_bounds__(xg_maxthr(Q), xg_minblk(Q))
   extern __shared__ __align__(16) unsigned char sraw[];
   __shared__ __align__(16) XgArgs s;
   const BatchItem w = xg_tile(s, p, insts, items, stage);
-  passA_g_tile<M, Q>(sraw, s, w.b, 2 * w.a);
+  passA_g_tile<M, Q>(sraw, s, blockIdx.z, w.b, 2 * w.a);
+}
+
+// The inverse x transforms of one component (blockIdx.z) of a row pair; the
+// demag field waits where the cell's stage derivative will be written.
+template <int M, int Q>
+__global__ void __launch_bounds__(xg_maxthr(Q), xg_minblk(Q)) k_invx_g(const __grid_constant__ XgArgs p) {
+  using X = Xg<M, Q>;
+  constexpr int N = X::N, LP = X::LP, HX = X::HX;
+  constexpr bool HALF = Q == 1;
+  static_assert(X::NB == 1, "one component per warp");
+  extern __shared__ __align__(16) unsigned char sraw[];
+  float4* G = reinterpret_cast<float4*>(sraw);   // [HX + 1]: (X_a, X_b); then the transforms' regions
+  float2* W = reinterpret_cast<float2*>(sraw);   // [Q][LP]
+  const Grid& g = p.g;
+  const int nx = g.nx, ny = g.ny, y0 = 2 * blockIdx.x, z = blockIdx.y, c = blockIdx.z;
+  const int lane = lane_id(), r = threadIdx.x >> 5;
+  const bool two = y0 + 1 < ny;
+  const long long kst = (long long)3 * g.nz * ny, t0 = ((long long)c * g.nz + z) * ny + y0;
+  const float2* T = p.d.T;
+  after_predecessor();
+  if (two && !(ny & 1) && !(reinterpret_cast<unsigned long long>(T) & 15)) {
+    for (int k = threadIdx.x; k <= HX; k += blockDim.x)
+      if (MMP_IN(g, t0 + k * kst + 1, g.lim_T)) cp_async16(G + k, T + t0 + k * kst);
+  } else {
+    for (int k = threadIdx.x; k <= HX; k += blockDim.x) {
+      if (!MMP_IN(g, t0 + k * kst + (two ? 1 : 0), g.lim_T)) continue;
+      cp_async8(reinterpret_cast<float2*>(G + k), T + t0 + k * kst);
+      if (two) cp_async8(reinterpret_cast<float2*>(G + k) + 1, T + t0 + k * kst + 1);
+      else reinterpret_cast<float2*>(G + k)[1] = make_float2(0.0f, 0.0f);
+    }
+  }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncthreads();
+  float2 v[M], o[32];
+  if (r < Q) {
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const int k = Q * (lane + 32 * m) + r;
+      const bool lo = k <= HX;
+      const float4 q = G[lo ? k : X::Px - k];
+      v[m] = lo ? make_float2(q.x - q.w, q.y + q.z) : make_float2(q.x + q.w, q.z - q.y);
+    }
+  }
+  __syncthreads();
+  float* out = p.f.kout + c * g.n + (long long)nx * (y0 + (long long)ny * z);
+  if (r < Q) {
+    float2* scr = W + r * LP;
+    gfft<M, 1, false, HALF, true>(v, o, scr, p.d.tw_wx);
+    if (lane < M) {
+#pragma unroll
+      for (int k2 = 0; k2 < (HALF ? 16 : 32); ++k2) {
+        const int x = lane + M * k2;
+        if (Q > 1) {
+          scr[x] = r ? cmul(o[k2], cconj(__ldg(p.d.tw_wx2 + r * x))) : o[k2];
+        } else if (x < nx && MMP_IN(g, (out - p.f.kout) + x, g.lim_state)) {
+          out[x] = o[k2].x;
+          if (two) out[nx + x] = o[k2].y;
+        }
+      }
+    }
+  }
+  if constexpr (Q > 1) {
+    __syncthreads();
+    auto put = [&](int x, float2 u) {
+      if (x >= nx || !MMP_IN(g, (out - p.f.kout) + x, g.lim_state)) return;
+      out[x] = u.x;
+      if (two) out[nx + x] = u.y;
+    };
+    for (int x = threadIdx.x; x < N; x += blockDim.x) {
+      const float2* t = W + x;
+      if constexpr (Q == 2) {
+        put(x, cadd(t[0], t[LP]));
+      } else {
+        const float2 e = cadd(t[0], t[2 * LP]), q = cadd(t[LP], t[3 * LP]);
+        const float2 em = csub(t[0], t[2 * LP]), qm = csub(t[LP], t[3 * LP]);
+        put(x, make_float2(e.x + q.x, e.y + q.y));
+        put(x + N, make_float2(em.x - qm.y, em.y + qm.x));   // + i (t1 - t3)
+      }
+    }
+  }
 }
 
 template <int M, int Q, int KIND>
@@ -426,7 +543,7 @@ cudaError_t launch_xg_t(int pass, int kind, const XgArgs& p, const XgLaunch& l, 
 template <typename K>
 static cudaError_t xg_go(K kernel, const XgArgs& p, const XgLaunch& l, const BatchInst* insts, const BatchItem* items,
                          int stage, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+  cudaError_t e = set_smem(kernel, l.smem, sizeof(XgArgs) + sizeof(RegionCoef) + 256);
   if (e != cudaSuccess) return e;
   if (!insts) return launch_chained(p.d.chain, kernel, l.grid, l.threads, l.smem, st, p, insts, items, stage);
   kernel<<<l.grid, l.threads, l.smem, st>>>(p, insts, items, stage);
@@ -436,12 +553,19 @@ template <int M, int Q>
 cudaError_t launch_xg_t(int pass, int kind, const XgArgs& p, const XgLaunch& l, const BatchInst* insts,
                         const BatchItem* items, int stage, cudaStream_t st) {
   if (pass == 0) return xg_go(k_passA_g<M, Q>, p, l, insts, items, stage, st);
-  switch (kind) {
-    case 0: return xg_go(k_passC_g<M, Q, 0>, p, l, insts, items, stage, st);
-    case 1: return xg_go(k_passC_g<M, Q, 1>, p, l, insts, items, stage, st);
-    case 2: return xg_go(k_passC_g<M, Q, 2>, p, l, insts, items, stage, st);
-    default: return xg_go(k_passC_g<M, Q, 3>, p, l, insts, items, stage, st);
+  if constexpr (M > 8) {
+    if (pass == 1) {
+      const cudaError_t e = set_smem(k_invx_g<M, Q>, l.smem);
+      return e != cudaSuccess ? e : launch_chained(p.d.chain, k_invx_g<M, Q>, l.grid, l.threads, l.smem, st, p);
+    }
   }
+  if (kind == 0) return xg_go(k_passC_g<M, Q, 0>, p, l, insts, items, stage, st);
+  if constexpr (M <= 8) {   // above, several regions or sublattices take k_invx_g and k_cells_g (xg_split)
+    if (kind == 1) return xg_go(k_passC_g<M, Q, 1>, p, l, insts, items, stage, st);
+    if (kind == 2) return xg_go(k_passC_g<M, Q, 2>, p, l, insts, items, stage, st);
+    return xg_go(k_passC_g<M, Q, 3>, p, l, insts, items, stage, st);
+  }
+  return cudaErrorInvalidValue;
 }
 #define MMP_XG(M, Q)                                                                                              \
   template cudaError_t launch_xg_t<M, Q>(int, int, const XgArgs&, const XgLaunch&, const BatchInst*,              \
