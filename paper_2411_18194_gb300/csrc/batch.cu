@@ -126,9 +126,11 @@ struct mmp_batch {
   std::vector<cudaEvent_t> join;
   bool list_valid = false;
   int sms = 0;
-  // fixed-step graph of one lock step over the current list
+  // graph of one lock step over the current list: the six stages, of fixed
+  // steps (graph_fixed) with the accept
   cudaGraphExec_t graph = nullptr;
-  bool graph_valid = false;
+  bool graph_valid = false, graph_fixed = false;
+  int list_attempts = 0;        // adaptive lock steps of the current list
   long long per_step = 0;       // kernel launches of one graph replay
   long long launches = 0;
   // tracing: events around every pass launch (lock steps then launch
@@ -358,6 +360,7 @@ int build_list(mmp_batch* b, const std::vector<int>& mem) {
   b->list = L;
   b->list_valid = true;
   b->graph_valid = false;
+  b->list_attempts = 0;
   return MMP_OK;
 }
 
@@ -422,6 +425,32 @@ int upload_insts(mmp_batch* b) {
   BCK(cudaMemcpyAsync(b->d_inst, b->h_inst.data(), b->h_inst.size() * sizeof(BatchInst), cudaMemcpyHostToDevice,
                       b->stream),
       "batch: upload descriptors");
+  return MMP_OK;
+}
+
+// The graph of one lock step over the current list.
+int ensure_graph(mmp_batch* b, bool fixed, int nact) {
+  if (b->graph_valid && b->graph_fixed == fixed) return MMP_OK;
+  if (b->graph) cudaGraphExecDestroy(b->graph);
+  b->graph = nullptr;
+  const long long before = b->launches;
+  BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeRelaxed), "batch: begin capture");
+  int rc = MMP_OK;
+  for (int s = 1; s <= 6 && rc == MMP_OK; ++s) rc = launch_stage(b, s);
+  if (rc == MMP_OK && fixed)
+    rc = launch_batch_accept(b->d_inst, nact, b->stream) == cudaSuccess ? MMP_OK
+                                                                        : cuda_fail(cudaGetLastError(), "batch: accept");
+  cudaGraph_t gr = nullptr;
+  cudaError_t e = cudaStreamEndCapture(b->stream, &gr);
+  b->per_step = b->launches - before + (fixed ? 1 : 0);
+  b->launches = before;
+  BTRY(rc);
+  BCK(e, "batch: end capture");
+  e = cudaGraphInstantiate(&b->graph, gr, 0);
+  cudaGraphDestroy(gr);
+  BCK(e, "batch: instantiate");
+  b->graph_valid = true;
+  b->graph_fixed = fixed;
   return MMP_OK;
 }
 
@@ -669,27 +698,7 @@ int advance_loop(mmp_batch* b, int max_attempts) {
       // whole lock steps from one graph: every member takes K steps
       long long K = max_attempts - attempts;
       for (int i : act) K = std::min(K, b->members[i].left);
-      if (!b->graph_valid) {
-        if (b->graph) cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-        const long long before = b->launches;
-        BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeRelaxed), "batch: begin capture");
-        int rc = MMP_OK;
-        for (int s = 1; s <= 6 && rc == MMP_OK; ++s) rc = launch_stage(b, s);
-        if (rc == MMP_OK) rc = launch_batch_accept(b->d_inst, (int)act.size(), b->stream) == cudaSuccess
-                                   ? MMP_OK
-                                   : cuda_fail(cudaGetLastError(), "batch: accept");
-        cudaGraph_t gr = nullptr;
-        cudaError_t e = cudaStreamEndCapture(b->stream, &gr);
-        b->per_step = b->launches - before + 1;
-        b->launches = before;
-        BTRY(rc);
-        BCK(e, "batch: end capture");
-        e = cudaGraphInstantiate(&b->graph, gr, 0);
-        cudaGraphDestroy(gr);
-        BCK(e, "batch: instantiate");
-        b->graph_valid = true;
-      }
+      BTRY(ensure_graph(b, true, (int)act.size()));
       for (long long s = 0; s < K; ++s) {
         BCK(cudaGraphLaunch(b->graph, b->stream), "batch: graph launch");
         b->launches += b->per_step;
@@ -707,7 +716,15 @@ int advance_loop(mmp_batch* b, int max_attempts) {
     }
     // one lock step with the errors read back
     BCK(cudaMemsetAsync(b->d_red, 0, 2 * act.size() * sizeof(unsigned), b->stream), "batch: reset errors");
-    for (int s = 1; s <= 6; ++s) BTRY(launch_stage(b, s));
+    // from the third lock step of a list on by its graph: one by one the launches
+    // and the events between side streams cost the host more than the kernels run
+    if (b->prof || ++b->list_attempts <= 2) {
+      for (int s = 1; s <= 6; ++s) BTRY(launch_stage(b, s));
+    } else {
+      BTRY(ensure_graph(b, false, (int)act.size()));
+      BCK(cudaGraphLaunch(b->graph, b->stream), "batch: graph launch");
+      b->launches += b->per_step;
+    }
     BCK(cudaMemcpyAsync(b->h_red, b->d_red, 2 * act.size() * sizeof(unsigned), cudaMemcpyDeviceToHost, b->stream),
         "batch: read errors");
     BCK(cudaStreamSynchronize(b->stream), "batch: sync");

@@ -22,10 +22,10 @@ cudaError_t launch_batch_passA(const BatchInst* insts, const BatchItem* items, i
                                size_t smem, cudaStream_t s) {
   cudaError_t e;
   if (stage == 0) {
-    if ((e = set_smem(k_batch_passA<false>, smem)) != cudaSuccess) return e;
+    if ((e = set_smem(k_batch_passA<false>, smem, 2048)) != cudaSuccess) return e;
     k_batch_passA<false><<<nitems, threads, smem, s>>>(insts, items, stage);
   } else {
-    if ((e = set_smem(k_batch_passA<true>, smem)) != cudaSuccess) return e;
+    if ((e = set_smem(k_batch_passA<true>, smem, 2048)) != cudaSuccess) return e;
     k_batch_passA<true><<<nitems, threads, smem, s>>>(insts, items, stage);
   }
   return cudaGetLastError();

@@ -49,9 +49,9 @@ struct mmp_ctx {
   float2 *d_tw_wx = nullptr, *d_tw_wx2 = nullptr;   // warp passes A and C (MMP_ENGINE_WARP_X)
   float* d_tw_tc = nullptr;    // tensor-core DFT32 matrices (MMP_ENGINE_TC_Y)
   unsigned* d_flag = nullptr;  // set by a device wait that ran past its limit
-  unsigned* d_red = nullptr;   // [0] error bits, [1] torque bits
+  unsigned* d_red = nullptr;   // [0] error bits, [1] torque bits, then the coefficients of an attempt
   double* d_energy = nullptr;  // [MMP_NTERMS] (mmp_energy)
-  unsigned* h_red = nullptr;   // pinned
+  unsigned* h_red = nullptr;   // pinned: [0, 2) read back, from 2 on the copy source of d_red
   int nparts = 0;              // 3-vectors in the state
   long long nstate = 0;        // floats in the state
   FftPlan plan_x{}, plan_ly{};
@@ -75,6 +75,17 @@ struct mmp_ctx {
   float* g_k0 = nullptr;
   double g_dt = 0.0;
   int g_method = -1, g_ks = 0;
+  // adaptive attempts (replay_attempt), one graph per side of the buffer swap
+  struct AttemptGraph {
+    cudaGraphExec_t exec = nullptr;
+    float* y = nullptr;
+    float* k0 = nullptr;
+    int method = -1, relax = 0;
+    long long gen = -1;
+  } ag[2];
+  long long ag_gen = -1;       // configuration whose attempts ag_seen counts
+  int ag_seen = 0;
+  bool ag_fresh = false;       // the graph stream follows the context's stream
   long long config_gen = 0, g_config_gen = -1;   // bumped by changes a graph would have baked in
   // tracing
   bool prof = false;

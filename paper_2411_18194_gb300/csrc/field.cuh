@@ -264,10 +264,12 @@ __device__ __forceinline__ void field_cell(const float* b3, const Grid& g, const
       f.kout[idx] = o.tau[i];
       if (f.Bout) f.Bout[idx] = o.B[i];
       if (f.err) {
-        float ev = f.ecoef[6] * o.tau[i];
+        float ev = error_coef_at(f, 6) * o.tau[i];
 #pragma unroll
-        for (int j = 0; j < 6; ++j)
-          if (f.ecoef[j] != 0.0f) ev = fmaf(f.ecoef[j], f.ek[j][idx], ev);
+        for (int j = 0; j < 6; ++j) {
+          const float ej = error_coef_at(f, j);
+          if (ej != 0.0f) ev = fmaf(ej, f.ek[j][idx], ev);
+        }
         ev = fabsf(ev);
         emax = isnan(ev) || ev > emax ? ev : emax;
       }

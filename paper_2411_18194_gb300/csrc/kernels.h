@@ -66,6 +66,7 @@ struct StageArgs {
   const float* y;            // state at the start of the step
   const float* k[7];         // previous stages (nk used)
   float coef[7];             // dt * a_ij (rounded from FP64)
+  const float* cdev;         // the same in device memory (captured attempts), or null
   int nk;
   int normalize;             // renormalise m (the 5th-order stage)
   float* stage;              // output stage state
@@ -115,10 +116,22 @@ struct FieldArgs {
   // error estimate of the 5th-order stage: err = max |sum_j e_j k_j|
   const float* ek[6];
   float ecoef[7];            // dt * (b_j - b*_j)
+  const float* cdev;         // the same in device memory (captured attempts), or null
   unsigned* err;             // atomicMax target (float bits)
   int relax;                 // damping-only torque (relax mode)
   unsigned* torque_max;      // max |m x B| (float bits) in relax mode
 };
+
+// Coefficients of the stage (read once into shared memory: a selection at every
+// use between the stage loads kept them from being in flight together, and cost a
+// fifth of pass A) and coefficient j of the error estimate.
+__device__ __forceinline__ void stage_coefs_load(const StageArgs& a, float* cf) {
+#pragma unroll
+  for (int j = 0; j < 7; ++j) cf[j] = a.cdev ? __ldg(a.cdev + j) : a.coef[j];
+}
+__device__ __forceinline__ float error_coef_at(const FieldArgs& f, int j) {
+  return f.cdev ? __ldg(f.cdev + j) : f.ecoef[j];
+}
 
 struct ElasticArgs {
   const float* stage;        // stage state (u, v at parts nsub, nsub+1)

@@ -37,6 +37,10 @@ int fail(int code, const char* fmt, ...) {
   return code;
 }
 
+// Words of mmp_ctx::d_red: error and torque bits, the stage coefficients
+// (stages 2 .. 7, seven each) and the error coefficients of an attempt.
+constexpr int kRedStage = 2, kRedError = kRedStage + 6 * 7, kRedWords = kRedError + 7;
+
 const double kRc = 10.0;   // Newell below 10 max(cell), asymptotic above
 
 float2 split(double v) {
@@ -564,7 +568,7 @@ struct Traced {
 // One field evaluation.  With `sa.y` set the stage is assembled from it
 // into ctx->d_stage; otherwise `src` (the current state) is evaluated.
 int evaluate(mmp_ctx* ctx, StageArgs sa, const float* src, float* kout, float* Bout, unsigned* err,
-             const float* ecoef, const float* const* ek, int relax, unsigned* tmax) {
+             const float* ecoef, const float* const* ek, int relax, unsigned* tmax, const float* ecdev = nullptr) {
   const Grid& g = ctx->g;
   const bool demag = has(ctx, MMP_T_DEMAG);
   const bool elastic = has(ctx, MMP_T_ELASTIC);
@@ -575,6 +579,17 @@ int evaluate(mmp_ctx* ctx, StageArgs sa, const float* src, float* kout, float* B
   sa.nparts = ctx->nparts;
   sa.nsub = ctx->nsub;
   const float* stage = sa.stage;
+  ElasticArgs ea;
+  ea.stage = stage;
+  ea.kout = kout;
+  ea.eps = ctx->d_eps;
+  ea.sig = ctx->d_sig;
+  ea.c11 = (float)ctx->glob[MMP_C11];
+  ea.c12 = (float)ctx->glob[MMP_C12];
+  ea.c44 = (float)ctx->glob[MMP_C44];
+  ea.eta = (float)ctx->glob[MMP_ETA];
+  ea.inv_rho = ctx->glob[MMP_RHO] > 0 ? (float)(1.0 / ctx->glob[MMP_RHO]) : 0.0f;
+  ea.terms = ctx->terms;
   const bool wx = demag && (ctx->engine & MMP_ENGINE_WARP_X);
   if (demag) {
     {
@@ -587,17 +602,6 @@ int evaluate(mmp_ctx* ctx, StageArgs sa, const float* src, float* kout, float* B
     Traced t(ctx, MMP_K_ASSEMBLE);
     CK(launch_assemble(g, sa, ctx->stream), "assemble");
   }
-  ElasticArgs ea;
-  ea.stage = stage;
-  ea.kout = kout;
-  ea.eps = ctx->d_eps;
-  ea.sig = ctx->d_sig;
-  ea.c11 = (float)ctx->glob[MMP_C11];
-  ea.c12 = (float)ctx->glob[MMP_C12];
-  ea.c44 = (float)ctx->glob[MMP_C44];
-  ea.eta = (float)ctx->glob[MMP_ETA];
-  ea.inv_rho = ctx->glob[MMP_RHO] > 0 ? (float)(1.0 / ctx->glob[MMP_RHO]) : 0.0f;
-  ea.terms = ctx->terms;
   if (strain) { Traced t(ctx, MMP_K_STRAIN); CK(launch_strain(g, ea, ctx->nsub, ctx->stream), "strain"); }
   FieldArgs f;
   memset(&f, 0, sizeof f);
@@ -610,6 +614,7 @@ int evaluate(mmp_ctx* ctx, StageArgs sa, const float* src, float* kout, float* B
   if (err) {
     for (int j = 0; j < 7; ++j) f.ecoef[j] = ecoef[j];
     for (int j = 0; j < 6; ++j) f.ek[j] = ek[j];
+    f.cdev = ecdev;
   }
   f.relax = relax;
   f.torque_max = tmax;
@@ -627,6 +632,15 @@ int evaluate(mmp_ctx* ctx, StageArgs sa, const float* src, float* kout, float* B
   return MMP_OK;
 }
 
+// The context's private stream and events for captured work.
+int graph_stream(mmp_ctx* ctx) {
+  if (ctx->gev[1]) return MMP_OK;
+  if (!ctx->gstream) CK(cudaStreamCreateWithFlags(&ctx->gstream, cudaStreamNonBlocking), "graph stream");
+  for (cudaEvent_t& ev : ctx->gev)
+    if (!ev) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "graph event");
+  return MMP_OK;
+}
+
 int ensure_k1(mmp_ctx* ctx, int relax) {
   if (ctx->k1_valid && ctx->k1_relax == relax) return MMP_OK;
   StageArgs sa;
@@ -637,18 +651,15 @@ int ensure_k1(mmp_ctx* ctx, int relax) {
   return MMP_OK;
 }
 
-// One attempt of size h of the context's method: stages 1..S, the last at
-// the renormalised solution (whose k is the next step's k1).  With want_err
-// the error estimate (and the torque maximum at the new state) are read
-// back (one synchronisation).
-int attempt(mmp_ctx* ctx, double h, bool want_err, int relax, double* err_out, double* tmax_out) {
-  TRY(ensure_k1(ctx, relax));
-  if (want_err) CK(cudaMemsetAsync(ctx->d_red, 0, 2 * sizeof(unsigned), ctx->stream), "reset error");
+// The kernels of one attempt of size h; with `dev` they read its coefficients
+// from d_red instead of their arguments (which h only has to fill).
+int attempt_stages(mmp_ctx* ctx, double h, bool want_err, int relax, bool dev) {
   const Tableau& T = tableau(ctx->method);
   float ecoef[7];
   error_coefs(T, h, ecoef);
   const float* ek[6];
   for (int j = 0; j < 6; ++j) ek[j] = j < T.S ? ctx->d_k[j] : nullptr;
+  const float* dred = reinterpret_cast<const float*>(ctx->d_red);
   for (int i = 1; i <= T.S; ++i) {
     StageArgs sa;
     memset(&sa, 0, sizeof sa);
@@ -656,15 +667,103 @@ int attempt(mmp_ctx* ctx, double h, bool want_err, int relax, double* err_out, d
     sa.nk = i;
     for (int j = 0; j < i; ++j) sa.k[j] = ctx->d_k[j];
     stage_coefs(T, h, i, sa.coef);
+    if (dev) sa.cdev = dred + kRedStage + 7 * (i - 1);
     sa.normalize = (i == T.S);
     bool last = (i == T.S);
     TRY(evaluate(ctx, sa, nullptr, ctx->d_k[i], nullptr, last && want_err ? ctx->d_red : nullptr, ecoef, ek,
-                 relax, last && want_err ? ctx->d_red + 1 : nullptr));
+                 relax, last && want_err ? ctx->d_red + 1 : nullptr, dev ? dred + kRedError : nullptr));
+  }
+  return MMP_OK;
+}
+
+// An adaptive attempt as one graph launch: the coefficients of its step size
+// and the cleared maxima copied from pinned memory, the kernels, the maxima
+// read back.  Launched one by one, the 18 or more kernels of an attempt cost the
+// host about 4 us each, more than most of them run at 512x512x1 and below.  A
+// configuration's first attempts are launched directly: a graph costs about as
+// much to make as two of them.  One graph for each side of the y/stage swap.
+int replay_attempt(mmp_ctx* ctx, double h, int relax) {
+  const Tableau& T = tableau(ctx->method);
+  float* hc = reinterpret_cast<float*>(ctx->h_red + 2);
+  memset(hc, 0, kRedWords * sizeof(float));
+  for (int i = 1; i <= T.S; ++i) stage_coefs(T, h, i, hc + kRedStage + 7 * (i - 1));
+  error_coefs(T, h, hc + kRedError);
+  TRY(graph_stream(ctx));
+  mmp_ctx::AttemptGraph* a = nullptr;
+  for (auto& c : ctx->ag)
+    if (c.exec && c.y == ctx->d_y && c.k0 == ctx->d_k[0] && c.method == ctx->method && c.relax == relax &&
+        c.gen == ctx->config_gen)
+      a = &c;
+  if (!a) {
+    a = &ctx->ag[0];
+    if (ctx->ag[0].exec && ctx->ag[0].gen == ctx->config_gen && ctx->ag[0].method == ctx->method &&
+        ctx->ag[0].relax == relax)
+      a = &ctx->ag[1];
+    if (a->exec) cudaGraphExecDestroy(a->exec);
+    a->exec = nullptr;
+    cudaStream_t user = ctx->stream;
+    ctx->stream = ctx->gstream;
+    cudaError_t e = cudaStreamBeginCapture(ctx->gstream, cudaStreamCaptureModeRelaxed);
+    int rc = e == cudaSuccess ? MMP_OK : cuda_check(ctx, e, "begin capture");
+    cudaGraph_t gr = nullptr;
+    if (rc == MMP_OK) {
+      e = cudaMemcpyAsync(ctx->d_red, ctx->h_red + 2, kRedWords * sizeof(unsigned), cudaMemcpyHostToDevice,
+                          ctx->gstream);
+      const long long evals = ctx->evals;
+      rc = attempt_stages(ctx, h, true, relax, true);
+      ctx->evals = evals;   // captured, not run
+      cudaError_t e2 = cudaMemcpyAsync(ctx->h_red, ctx->d_red, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost,
+                                       ctx->gstream);
+      if (e == cudaSuccess) e = e2;
+      e2 = cudaStreamEndCapture(ctx->gstream, &gr);
+      if (e == cudaSuccess) e = e2;
+    }
+    ctx->stream = user;
+    TRY(rc);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&a->exec, gr, 0);
+    if (gr) cudaGraphDestroy(gr);
+    CK(e, "capture attempt");
+    a->y = ctx->d_y;
+    a->k0 = ctx->d_k[0];
+    a->method = ctx->method;
+    a->relax = relax;
+    a->gen = ctx->config_gen;
+  }
+  if (!ctx->ag_fresh) {   // after the work already queued on the context's stream
+    CK(cudaEventRecord(ctx->gev[0], ctx->stream), "graph event");
+    CK(cudaStreamWaitEvent(ctx->gstream, ctx->gev[0], 0), "graph wait");
+    ctx->ag_fresh = true;
+  }
+  CK(cudaGraphLaunch(a->exec, ctx->gstream), "graph launch");
+  ctx->evals += T.S;
+  CK(cudaStreamSynchronize(ctx->gstream), "sync");
+  return MMP_OK;
+}
+
+// One attempt of size h of the context's method: stages 1..S, the last at
+// the renormalised solution (whose k is the next step's k1).  With want_err
+// the error estimate (and the torque maximum at the new state) are read
+// back (one synchronisation).
+int attempt(mmp_ctx* ctx, double h, bool want_err, int relax, double* err_out, double* tmax_out) {
+  TRY(ensure_k1(ctx, relax));
+  if (ctx->ag_gen != ctx->config_gen) {
+    ctx->ag_gen = ctx->config_gen;
+    ctx->ag_seen = 0;
+  }
+  const bool graph = want_err && !ctx->prof && ctx->ag_seen >= 4;
+  if (want_err) ctx->ag_seen += ctx->ag_seen < 4;
+  if (graph) {
+    TRY(replay_attempt(ctx, h, relax));
+  } else {
+    if (want_err) CK(cudaMemsetAsync(ctx->d_red, 0, 2 * sizeof(unsigned), ctx->stream), "reset error");
+    TRY(attempt_stages(ctx, h, want_err, relax, false));
+    if (want_err) {
+      CK(cudaMemcpyAsync(ctx->h_red, ctx->d_red, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream),
+         "read error");
+      CK(cudaStreamSynchronize(ctx->stream), "sync");
+    }
   }
   if (want_err) {
-    CK(cudaMemcpyAsync(ctx->h_red, ctx->d_red, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream),
-       "read error");
-    CK(cudaStreamSynchronize(ctx->stream), "sync");
     float e, tm;
     memcpy(&e, &ctx->h_red[0], 4);
     memcpy(&tm, &ctx->h_red[1], 4);
@@ -693,11 +792,7 @@ int replay_pairs(mmp_ctx* ctx, long long pairs) {
   const Tableau& T = tableau(ctx->method);
   const bool same = ctx->gexec && ctx->g_y == ctx->d_y && ctx->g_k0 == ctx->d_k[0] && ctx->g_dt == ctx->dt &&
                     ctx->g_method == ctx->method && ctx->g_config_gen == ctx->config_gen && ctx->g_ks == T.S;
-  if (!ctx->gstream) {
-    CK(cudaStreamCreateWithFlags(&ctx->gstream, cudaStreamNonBlocking), "graph stream");
-    CK(cudaEventCreateWithFlags(&ctx->gev[0], cudaEventDisableTiming), "graph event");
-    CK(cudaEventCreateWithFlags(&ctx->gev[1], cudaEventDisableTiming), "graph event");
-  }
+  TRY(graph_stream(ctx));
   if (!same) {
     if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
     ctx->gexec = nullptr;
@@ -743,6 +838,7 @@ int replay_pairs(mmp_ctx* ctx, long long pairs) {
 int advance(mmp_ctx* ctx, long long nsteps, double until, int relax, double torque_tol, double timeout_s,
             bool* converged) {
   TRY(prepare(ctx));
+  ctx->ag_fresh = false;
   auto t0 = std::chrono::steady_clock::now();
   long long done = 0;
   const bool adaptive = ctx->adaptive || relax;
@@ -897,7 +993,7 @@ int mmp_create(mmp_ctx** out, int nx, int ny, int nz, double cx, double cy, doub
   int rc = MMP_OK;
 #define CR(x) do { if (rc == MMP_OK) rc = (x); } while (0)
   CR(alloc_into(ctx, ctx->d_coef, 2 * MMP_MAX_REGIONS * sizeof(RegionCoef)));
-  CR(alloc_into(ctx, ctx->d_red, 2 * sizeof(unsigned)));
+  CR(alloc_into(ctx, ctx->d_red, kRedWords * sizeof(unsigned)));
   CR(alloc_into(ctx, ctx->d_flag, sizeof(unsigned)));
   if (rc == MMP_OK && cudaMemset(ctx->d_flag, 0, sizeof(unsigned)) != cudaSuccess)
     rc = cuda_check(ctx, cudaGetLastError(), "clear device flag");
@@ -907,7 +1003,7 @@ int mmp_create(mmp_ctx** out, int nx, int ny, int nz, double cx, double cy, doub
   g.lim_B = 3LL * nsub * n;
   g.lim_T = (long long)g.kxn * 3 * g.nz * g.ny;
   g.lim_khat = (long long)g.kxn * g.kyn * g.krow;
-  if (rc == MMP_OK && cudaMallocHost(&ctx->h_red, 2 * sizeof(unsigned)) != cudaSuccess) {
+  if (rc == MMP_OK && cudaMallocHost(&ctx->h_red, (2 + kRedWords) * sizeof(unsigned)) != cudaSuccess) {
     cudaGetLastError();
     rc = fail(MMP_E_OOM, "pinned allocation failed");
   }
@@ -951,6 +1047,8 @@ int mmp_destroy(mmp_ctx* ctx) {
   cudaStreamSynchronize(ctx->stream);
   release_khat(ctx);
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
+  for (auto& a : ctx->ag)
+    if (a.exec) cudaGraphExecDestroy(a.exec);
   if (ctx->gstream) cudaStreamDestroy(ctx->gstream);
   for (cudaEvent_t ev : ctx->gev)
     if (ev) cudaEventDestroy(ev);

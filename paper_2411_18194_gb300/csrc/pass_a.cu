@@ -59,7 +59,7 @@ cudaError_t launch_passA(const Grid& g, const StageArgs& a, const DemagArgs& d, 
   cudaError_t e;
 #define MMP_PA(NS, AS)                                                      \
   do {                                                                      \
-    if ((e = set_smem(k_passA<NS, AS>, smem_passA(g) + 2 * g.ty * g.nx * sizeof(float))) != cudaSuccess) \
+    if ((e = set_smem(k_passA<NS, AS>, smem_passA(g) + 2 * g.ty * g.nx * sizeof(float), 64)) != cudaSuccess) \
       return e;                                                             \
     k_passA<NS, AS><<<grid, threads, sm, s>>>(g, a, d, c);                 \
   } while (0)

@@ -25,17 +25,17 @@ __host__ __device__ __forceinline__ size_t passa_inv_offset(int Px, int ty, int 
 }
 
 // Stage value of component c of part p at a cell: assembled from y and the
-// previous stages (ASSEMBLE) or read from the given stage state.
+// previous stages with the coefficients cf (ASSEMBLE) or read from the given stage state.
 template <bool ASSEMBLE>
-__device__ __forceinline__ float stage_value(const Grid& g, const StageArgs& a, long long n, int p, int c,
-                                             long long cell) {
+__device__ __forceinline__ float stage_value(const Grid& g, const StageArgs& a, const float* cf, long long n, int p,
+                                             int c, long long cell) {
   const long long idx = (long long)(3 * p + c) * n + cell;
   if (!MMP_IN(g, idx, g.lim_state)) return 0.0f;
   if (!ASSEMBLE) return a.stage[idx];
   float acc = a.y[idx];
 #pragma unroll
   for (int j = 0; j < 7; ++j)
-    if (j < a.nk) acc = fmaf(a.coef[j], a.k[j][idx], acc);
+    if (j < a.nk) acc = fmaf(cf[j], a.k[j][idx], acc);
   return acc;
 }
 
@@ -48,7 +48,7 @@ __device__ __forceinline__ float stage_value(const Grid& g, const StageArgs& a, 
 template <int NSUB, bool ASSEMBLE>
 __device__ __forceinline__ void passA_components(int c0, int nc, float2* fbuf, const float2* tw, const float* inv,
                                                  const Grid& g, const StageArgs& a, const DemagArgs& d,
-                                                 const Coefs& co, int z, int y0) {
+                                                 const Coefs& co, const float* cf, int z, int y0) {
   if (nc == 0) return;
   const int nx = g.nx, ny = g.ny, Px = g.Px;
   const int pitch = fft_pitch(Px);
@@ -81,7 +81,7 @@ __device__ __forceinline__ void passA_components(int c0, int nc, float2* fbuf, c
         const bool ok = e < total && x < nx && y < ny;
         cl[u][h] = ok ? x + (long long)nx * (y + (long long)ny * z) : -1;
 #pragma unroll
-        for (int s = 0; s < NSUB; ++s) mv[u][h][s] = ok ? stage_value<ASSEMBLE>(g, a, n, s, c, cl[u][h]) : 0.0f;
+        for (int s = 0; s < NSUB; ++s) mv[u][h][s] = ok ? stage_value<ASSEMBLE>(g, a, cf, n, s, c, cl[u][h]) : 0.0f;
       }
     }
 #pragma unroll
@@ -142,6 +142,9 @@ __device__ __forceinline__ void passA_tile(unsigned char* sraw, const Grid& g, c
   float2* tw = reinterpret_cast<float2*>(sraw + passa_twiddle_offset(Px, g.ty, g.xb));
   float* inv = reinterpret_cast<float*>(sraw + passa_inv_offset(Px, g.ty, g.xb));
   const long long n = g.n;
+  __shared__ float cf[7];
+  if (threadIdx.x == 0) stage_coefs_load(a, cf);
+  __syncthreads();
   for (int i = threadIdx.x; i < Px; i += blockDim.x) tw[i] = __ldg(d.tw_x + i);
   if (ASSEMBLE && (a.normalize || a.nparts > a.nsub)) {
     for (int e = threadIdx.x; e < g.ty * nx; e += blockDim.x) {
@@ -151,9 +154,9 @@ __device__ __forceinline__ void passA_tile(unsigned char* sraw, const Grid& g, c
       if (a.normalize) {
         // 1/|m_i| of the renormalised stage, per sublattice
         for (int s = 0; s < NSUB; ++s) {
-          float v0 = stage_value<true>(g, a, n, s, 0, cell);
-          float v1 = stage_value<true>(g, a, n, s, 1, cell);
-          float v2 = stage_value<true>(g, a, n, s, 2, cell);
+          float v0 = stage_value<true>(g, a, cf, n, s, 0, cell);
+          float v1 = stage_value<true>(g, a, cf, n, s, 1, cell);
+          float v2 = stage_value<true>(g, a, cf, n, s, 2, cell);
           float nn = v0 * v0 + v1 * v1 + v2 * v2;
           inv[(s * g.ty + row) * nx + x] = nn > 0.0f ? rnorm3df(v0, v1, v2) : 1.0f;
         }
@@ -162,7 +165,7 @@ __device__ __forceinline__ void passA_tile(unsigned char* sraw, const Grid& g, c
       for (int p = a.nsub; p < a.nparts; ++p)
         for (int c = 0; c < 3; ++c) {
           const long long idx = (long long)(3 * p + c) * n + cell;
-          if (MMP_IN(g, idx, g.lim_state)) a.stage[idx] = stage_value<true>(g, a, n, p, c, cell);
+          if (MMP_IN(g, idx, g.lim_state)) a.stage[idx] = stage_value<true>(g, a, cf, n, p, c, cell);
         }
     }
   }
@@ -170,9 +173,9 @@ __device__ __forceinline__ void passA_tile(unsigned char* sraw, const Grid& g, c
   // straight-line calls (a loop around the FFT body makes the compiler cut
   // the registers and spill); with xb = 3 the first call does all three
   const int rest = g.xb == 3 ? 0 : 1;
-  passA_components<NSUB, ASSEMBLE>(0, g.xb == 3 ? 3 : 1, fbuf, tw, inv, g, a, d, co, z, y0);
-  passA_components<NSUB, ASSEMBLE>(1, rest, fbuf, tw, inv, g, a, d, co, z, y0);
-  passA_components<NSUB, ASSEMBLE>(2, rest, fbuf, tw, inv, g, a, d, co, z, y0);
+  passA_components<NSUB, ASSEMBLE>(0, g.xb == 3 ? 3 : 1, fbuf, tw, inv, g, a, d, co, cf, z, y0);
+  passA_components<NSUB, ASSEMBLE>(1, rest, fbuf, tw, inv, g, a, d, co, cf, z, y0);
+  passA_components<NSUB, ASSEMBLE>(2, rest, fbuf, tw, inv, g, a, d, co, cf, z, y0);
 }
 
 }  // namespace mmp

@@ -6,6 +6,8 @@
 namespace mmp {
 
 __device__ __forceinline__ void assemble_cell(const Grid& g, const StageArgs& a, long long n, long long cell) {
+  float cf[7];
+  stage_coefs_load(a, cf);
   for (int p = 0; p < a.nparts; ++p) {
     float v[3];
 #pragma unroll
@@ -15,7 +17,7 @@ __device__ __forceinline__ void assemble_cell(const Grid& g, const StageArgs& a,
       float acc = a.y[idx];
 #pragma unroll
       for (int j = 0; j < 7; ++j)
-        if (j < a.nk) acc = fmaf(a.coef[j], a.k[j][idx], acc);
+        if (j < a.nk) acc = fmaf(cf[j], a.k[j][idx], acc);
       v[c] = acc;
     }
     if (a.normalize && p < a.nsub) {

@@ -65,10 +65,12 @@ __device__ __forceinline__ float4 st4_get(const float (&d)[4]) { return make_flo
 // Outputs of one cell: the stage derivative, B (optional), the error
 // estimate of the 5th-order stage and the torque maximum (both NaN-keeping).
 __device__ __forceinline__ void st4_errmax(const FieldArgs& f, long long idx, float tau, float& emax) {
-  float ev = f.ecoef[6] * tau;
+  float ev = error_coef_at(f, 6) * tau;
 #pragma unroll
-  for (int j = 0; j < 6; ++j)
-    if (f.ecoef[j] != 0.0f) ev = fmaf(f.ecoef[j], f.ek[j][idx], ev);
+  for (int j = 0; j < 6; ++j) {
+    const float ej = error_coef_at(f, j);
+    if (ej != 0.0f) ev = fmaf(ej, f.ek[j][idx], ev);
+  }
   ev = fabsf(ev);
   emax = isnan(ev) || ev > emax ? ev : emax;
 }

@@ -385,6 +385,10 @@ __device__ __forceinline__ BatchItem xg_tile(XgArgs& s, const XgArgs& p, const B
     xg_copy(s, p);
     after_predecessor();
     __syncthreads();
+    if (p.a.cdev) {   // a captured attempt: this step's coefficients
+      if (threadIdx.x < 7) s.a.coef[threadIdx.x] = __ldg(p.a.cdev + threadIdx.x);
+      __syncthreads();
+    }
     return BatchItem{0, (int)blockIdx.x, (int)blockIdx.y};
   }
   const BatchItem w = items[blockIdx.x];
@@ -413,6 +417,8 @@ __device__ __forceinline__ BatchItem xg_tile(XgArgs& s, const XgArgs& p, const B
       s.f.stage = st;
     } else if (j == 8) {
       s.a.nk = stage;
+      s.a.cdev = nullptr;
+      s.f.cdev = nullptr;
       s.a.normalize = last;
       s.a.nparts = 1;
       s.a.nsub = 1;

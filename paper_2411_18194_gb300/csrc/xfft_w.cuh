@@ -47,8 +47,8 @@ __host__ __device__ constexpr size_t field_w_smem() { return (size_t)3 * (kXwN +
 // ------------------------------------------------------------- pass A ----
 // Stage value of part p, component c at 4 consecutive cells (16-byte loads).
 template <bool ASSEMBLE>
-__device__ __forceinline__ float4 stage_value4(const Grid& g, const StageArgs& a, long long n, int p, int c,
-                                               long long cell) {
+__device__ __forceinline__ float4 stage_value4(const Grid& g, const StageArgs& a, const float* cf, long long n,
+                                               int p, int c, long long cell) {
   const long long idx = (long long)(3 * p + c) * n + cell;
   if (!MMP_IN(g, idx + 3, g.lim_state)) return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   if (!ASSEMBLE) return *reinterpret_cast<const float4*>(a.stage + idx);
@@ -57,7 +57,7 @@ __device__ __forceinline__ float4 stage_value4(const Grid& g, const StageArgs& a
   for (int j = 0; j < 7; ++j)
     if (j < a.nk) {
       const float4 k = __ldcs(reinterpret_cast<const float4*>(a.k[j] + idx));
-      const float cj = a.coef[j];
+      const float cj = cf[j];
       acc.x = fmaf(cj, k.x, acc.x);
       acc.y = fmaf(cj, k.y, acc.y);
       acc.z = fmaf(cj, k.z, acc.z);
@@ -70,8 +70,8 @@ __device__ __forceinline__ float4 stage_value4(const Grid& g, const StageArgs& a
 // 16-byte loads when nx is a multiple of 4, else V = 1), all parts, the
 // stage state written once, M_c = sum_s Ms m_s into Zin[c][x].h.
 template <int NSUB, bool ASSEMBLE, int V>
-__device__ __forceinline__ void passA_w_cells(const Grid& g, const StageArgs& a, const Coefs& co, float2* Zin,
-                                              int h, int x0, long long cell0) {
+__device__ __forceinline__ void passA_w_cells(const Grid& g, const StageArgs& a, const Coefs& co,
+                                              const float* cf, float2* Zin, int h, int x0, long long cell0) {
   const long long n = g.n;
   float Mv[3][V];
 #pragma unroll
@@ -84,10 +84,10 @@ __device__ __forceinline__ void passA_w_cells(const Grid& g, const StageArgs& a,
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       if constexpr (V == 4) {
-        const float4 q = stage_value4<ASSEMBLE>(g, a, n, s, c, cell0);
+        const float4 q = stage_value4<ASSEMBLE>(g, a, cf, n, s, c, cell0);
         m[c][0] = q.x; m[c][1] = q.y; m[c][2] = q.z; m[c][3] = q.w;
       } else {
-        m[c][0] = stage_value<ASSEMBLE>(g, a, n, s, c, cell0);
+        m[c][0] = stage_value<ASSEMBLE>(g, a, cf, n, s, c, cell0);
       }
     }
     if (ASSEMBLE && a.normalize) {
@@ -125,8 +125,8 @@ __device__ __forceinline__ void passA_w_cells(const Grid& g, const StageArgs& a,
         const long long idx = (long long)(3 * p + c) * n + cell0;
         if (!MMP_IN(g, idx + V - 1, g.lim_state)) continue;
         float* dst = a.stage + idx;
-        if constexpr (V == 4) *reinterpret_cast<float4*>(dst) = stage_value4<true>(g, a, n, p, c, cell0);
-        else dst[0] = stage_value<true>(g, a, n, p, c, cell0);
+        if constexpr (V == 4) *reinterpret_cast<float4*>(dst) = stage_value4<true>(g, a, cf, n, p, c, cell0);
+        else dst[0] = stage_value<true>(g, a, cf, n, p, c, cell0);
       }
   }
   float* Zf = reinterpret_cast<float*>(Zin);
@@ -136,19 +136,13 @@ __device__ __forceinline__ void passA_w_cells(const Grid& g, const StageArgs& a,
     for (int i = 0; i < V; ++i) Zf[2 * (c * kXwN + x0 + i) + h] = Mv[c][i];
 }
 
-// a.k[j], a.coef[j] for a run-time j by selects (an indexed parameter array
+// a.k[j] for a run-time j by selects (an indexed parameter array
 // would be copied to local memory)
 __device__ __forceinline__ const float* stage_k(const StageArgs& a, int j) {
   const float* p = a.k[0];
 #pragma unroll
   for (int i = 1; i < 7; ++i) p = j == i ? a.k[i] : p;
   return p;
-}
-__device__ __forceinline__ float stage_coef(const StageArgs& a, int j) {
-  float c = a.coef[0];
-#pragma unroll
-  for (int i = 1; i < 7; ++i) c = j == i ? a.coef[i] : c;
-  return c;
 }
 
 // Stage assembly of the tile's two rows with the stage vectors streamed
@@ -161,7 +155,8 @@ __device__ __forceinline__ float stage_coef(const StageArgs& a, int j) {
 // written once, and M = Ms m into Zin.
 template <bool ASSEMBLE>
 __device__ __forceinline__ void passA_w_assemble_async(float* buf0, float* buf1, float2* Zin, const Grid& g,
-                                                       const StageArgs& a, const Coefs& co, int z, int y0) {
+                                                       const StageArgs& a, const Coefs& co, const float* cf, int z,
+                                                       int y0) {
   constexpr int N = kXwN, IT = 3;   // at most 3 items of 4 cells per thread (2 rows x N / 4 / 192)
   const int nx = g.nx, ny = g.ny, q = nx >> 2;
   const long long n = g.n;
@@ -187,7 +182,7 @@ __device__ __forceinline__ void passA_w_assemble_async(float* buf0, float* buf1,
     else cp_async_wait_all();
     __syncthreads();
     float* b = (v & 1) ? buf1 : buf0;
-    const float cv = v == 0 ? 1.0f : stage_coef(a, v - 1);
+    const float cv = v == 0 ? 1.0f : cf[v - 1];
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
       const int e = threadIdx.x + it * kXwThreads;
@@ -259,16 +254,19 @@ __device__ __forceinline__ void passA_w_tile(unsigned char* sraw, const Grid& g,
   float2* Sodd = Zin + 3 * N;                      // [3][N] odd warps' scratch
   const float2* twT = d.tw_wx;                     // [N], global (L1)
   const int lane = lane_id(), warp = threadIdx.x >> 5;
+  __shared__ float cf[7];
+  if (threadIdx.x == 0) stage_coefs_load(a, cf);
+  __syncthreads();
   // 1. stage assembly of both rows into Zin (zero for x >= nx and a row y >= ny)
   if (NSUB == 1 && (nx & 3) == 0 && a.nparts == a.nsub) {
     passA_w_assemble_async<ASSEMBLE>(reinterpret_cast<float*>(Zin), reinterpret_cast<float*>(Sodd), Zin, g, a, co,
-                                     z, y0);
+                                     cf, z, y0);
   } else if ((nx & 3) == 0) {
     const int q = nx >> 2;
     for (int e = threadIdx.x; e < 2 * q; e += kXwThreads) {
       const int h = e >= q, x0 = 4 * (e - h * q), y = y0 + h;
       if (y < ny) {
-        passA_w_cells<NSUB, ASSEMBLE, 4>(g, a, co, Zin, h, x0, x0 + (long long)nx * (y + (long long)ny * z));
+        passA_w_cells<NSUB, ASSEMBLE, 4>(g, a, co, cf, Zin, h, x0, x0 + (long long)nx * (y + (long long)ny * z));
       } else {
         float* Zf = reinterpret_cast<float*>(Zin);
         for (int c = 0; c < 3; ++c)
@@ -279,7 +277,7 @@ __device__ __forceinline__ void passA_w_tile(unsigned char* sraw, const Grid& g,
     for (int e = threadIdx.x; e < 2 * nx; e += kXwThreads) {
       const int h = e >= nx, x0 = e - h * nx, y = y0 + h;
       if (y < ny) {
-        passA_w_cells<NSUB, ASSEMBLE, 1>(g, a, co, Zin, h, x0, x0 + (long long)nx * (y + (long long)ny * z));
+        passA_w_cells<NSUB, ASSEMBLE, 1>(g, a, co, cf, Zin, h, x0, x0 + (long long)nx * (y + (long long)ny * z));
       } else {
         float* Zf = reinterpret_cast<float*>(Zin);
         for (int c = 0; c < 3; ++c) Zf[2 * (c * N + x0) + h] = 0.0f;

@@ -1,0 +1,92 @@
+"""GPU: the forms of one computation that differ only in how it is launched are
+bitwise equal: adaptive attempts from a graph and one by one (tracing launches
+one by one), of a context and of a batch; and a batch member whose pass C is
+one kernel with its own context, where the inverse x transforms and the local
+field are two kernels."""
+import numpy as np
+import pytest
+
+from gpu_util import make_magnet
+from inputs import Problem, random_unit_vectors, stable_dt
+
+pytestmark = pytest.mark.gpu
+
+
+def _magnet(shape, seed, alpha=0.3):
+    p = Problem(shape, (4e-9, 4e-9, 2e-9), 1, frozenset({"DEMAG", "EXCH", "ZEEMAN"}))
+    p.set("MS", 8e5).set("AEX", 1.3e-11).set("ALPHA", alpha).set("B_EXT", (0.02, 0.0, 0.03))
+    return p, make_magnet(p, [random_unit_vectors(seed, shape)])
+
+
+def _m(mag):
+    import torch
+    nx, ny, nz = mag.shape
+    out = torch.empty((3, nz, ny, nx), dtype=torch.float32, device="cuda")
+    mag.get_m(0, out)
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("shape", [(48, 40, 1), (200, 24, 2), (1000, 16, 1), (1100, 10, 1), (7, 40, 2)])
+@pytest.mark.parametrize("method", ["DP45", "BS23"])
+def test_adaptive_graph_equals_direct_launches(shape, method):
+    res = []
+    for traced in (False, True):
+        p, mag = _magnet(shape, 11)
+        mag.set_solver(adaptive=True, dt=2e-14, tol=1e-5, method=method)
+        if traced:
+            mag.profile(True)
+        mag.step(7)          # the graph from the fifth attempt on
+        mag.step(6)          # captured before, both sides of the buffer swap
+        mag.set_param("ALPHA", 0.2, 0, -1)
+        mag.step(3)          # the coefficients' contents change, the graph stays
+        t = mag.time()
+        res.append((_m(mag), t["t"], t["dt"], t["steps"], t["rejected"], t["evals"]))
+        mag.close()
+    assert np.array_equal(res[0][0], res[1][0])
+    assert res[0][1:] == res[1][1:]
+
+
+def test_adaptive_graph_two_sublattices():
+    from inputs import config_small
+    w = config_small((1000, 6, 1), (2e-9, 2e-9, 2e-9), 5, terms=("DEMAG", "EXCH", "ANIS", "AFM", "MEL", "ELASTIC"), n_sub=2)
+    w.problem.glob.update(ETA=1e-15)
+    res = []
+    for traced in (False, True):
+        mag = make_magnet(w.problem, w.m0)
+        mag.set_solver(adaptive=True, dt=1e-15, tol=1e-4)
+        if traced:
+            mag.profile(True)
+        mag.step(12)
+        res.append((_m(mag), mag.time()))
+        mag.close()
+    assert np.array_equal(res[0][0], res[1][0])
+    assert res[0][1] == res[1][1]
+
+
+def test_batch_graph_and_split_pass_c_equal_solo():
+    import paper_2411_18194_gb300 as pkg
+    shapes = [(200, 30, 1), (300, 20, 2), (500, 9, 1), (700, 12, 1), (64, 64, 1), (1200, 6, 1)]
+    solo = []
+    for i, sh in enumerate(shapes):
+        p, mag = _magnet(sh, 40 + i)
+        mag.set_shape(R=1, stage_kernel=0, engine=0)
+        mag.set_solver(adaptive=True, dt=2e-14, tol=1e-5)
+        mag.run(3e-13)
+        solo.append((_m(mag), [mag.time()[k] for k in ("t", "dt", "steps", "rejected")]))
+        mag.close()
+    for traced in (False, True):
+        mags = []
+        with pkg.Batch() as b:
+            for i, sh in enumerate(shapes):
+                p, mag = _magnet(sh, 40 + i)
+                mag.set_shape(R=1, stage_kernel=0, engine=0)
+                mag.set_solver(adaptive=True, dt=2e-14, tol=1e-5)
+                mags.append(mag)
+                b.add(mag, "run", 3e-13)
+            if traced:
+                b.profile(True)
+            b.advance()
+        for mag, (m, t) in zip(mags, solo):
+            assert np.array_equal(_m(mag), m)
+            assert [mag.time()[k] for k in ("t", "dt", "steps", "rejected")] == t
+            mag.close()
