@@ -75,6 +75,9 @@ struct mmp_ctx {
   float* g_k0 = nullptr;
   double g_dt = 0.0;
   int g_method = -1, g_ks = 0;
+  // side stream of the elastic kernels (evaluate); events: after pass A, strain, force
+  cudaStream_t estream = nullptr;
+  cudaEvent_t eev[3] = {nullptr, nullptr, nullptr};
   // adaptive attempts (replay_attempt), one graph per side of the buffer swap
   struct AttemptGraph {
     cudaGraphExec_t exec = nullptr;
