@@ -129,6 +129,10 @@ __device__ __forceinline__ void stage_coefs_load(const StageArgs& a, float* cf) 
 #pragma unroll
   for (int j = 0; j < 7; ++j) cf[j] = a.cdev ? __ldg(a.cdev + j) : a.coef[j];
 }
+__device__ __forceinline__ void error_coefs_load(const FieldArgs& f, float* ec) {
+#pragma unroll
+  for (int j = 0; j < 7; ++j) ec[j] = f.cdev ? __ldg(f.cdev + j) : f.ecoef[j];
+}
 __device__ __forceinline__ float error_coef_at(const FieldArgs& f, int j) {
   return f.cdev ? __ldg(f.cdev + j) : f.ecoef[j];
 }
@@ -230,12 +234,16 @@ __host__ __device__ constexpr size_t xg_gather_bytes(int M, int Q) {
                                                                           : (size_t)24 * Q * xg_pitch(M, Q);
 }
 __host__ __device__ constexpr int xg_maxthr(int Q) { return Q == 4 ? 384 : 256; }
+// 128 registers a thread: at 80 (three blocks of 256 threads) the stage loads of
+// pass A are no longer all in flight and pass C's four-cell items spill; 512x512x4
+// four steps 2780 -> 2972 us (pass A at 80) -> 3124 (both), 1024x256x1
+// antiferromagnet 2665 -> 2873.
 __host__ __device__ constexpr int xg_minblk(int Q) { return Q == 4 ? 1 : 2; }
 // M and Q of the grid; false outside the engine (Px < 64).
 bool xg_shape(const Grid& g, int* M, int* Q);
 // Threads and dynamic shared memory of pass 0 (A) or 2 (C); cells: pass C
 // works cell by cell.
-struct XgPlan { int threads; size_t smem; };
+struct XgPlan { int threads; size_t smem; int v; };
 XgPlan xg_plan(const Grid& g, int pass, bool cells, bool batch);
 // Whether pass C is two kernels for this grid and kind.
 bool xg_split(const Grid& g, int kind);

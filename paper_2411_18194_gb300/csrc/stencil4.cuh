@@ -57,20 +57,52 @@ __device__ __forceinline__ float st4_fin(df a, float F) {
   const df w = two_sum(a.hi, F);
   return w.hi + (a.lo + w.lo);
 }
-__device__ __forceinline__ void st4_put(float (&d)[4], float4 q) {
-  d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
+// V consecutive floats (V = 1, 2 or 4; p aligned to them): read, read through the
+// read-only path, write.
+template <int V>
+__device__ __forceinline__ void st4_read(float (&d)[V], const float* p) {
+  if constexpr (V == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
+  } else if constexpr (V == 2) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    d[0] = q.x; d[1] = q.y;
+  } else {
+    d[0] = *p;
+  }
 }
-__device__ __forceinline__ float4 st4_get(const float (&d)[4]) { return make_float4(d[0], d[1], d[2], d[3]); }
+template <int V>
+__device__ __forceinline__ void st4_ldg(float (&d)[V], const float* p) {
+  if constexpr (V == 4) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+    d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
+  } else if constexpr (V == 2) {
+    const float2 q = __ldg(reinterpret_cast<const float2*>(p));
+    d[0] = q.x; d[1] = q.y;
+  } else {
+    d[0] = __ldg(p);
+  }
+}
+template <int V>
+__device__ __forceinline__ void st4_copy(float (&d)[V], const float (&q)[V]) {
+#pragma unroll
+  for (int j = 0; j < V; ++j) d[j] = q[j];
+}
+template <int V>
+__device__ __forceinline__ void st4_write(float* p, const float (&d)[V]) {
+  if constexpr (V == 4) *reinterpret_cast<float4*>(p) = make_float4(d[0], d[1], d[2], d[3]);
+  else if constexpr (V == 2) *reinterpret_cast<float2*>(p) = make_float2(d[0], d[1]);
+  else *p = d[0];
+}
 
 // Outputs of one cell: the stage derivative, B (optional), the error
 // estimate of the 5th-order stage and the torque maximum (both NaN-keeping).
-__device__ __forceinline__ void st4_errmax(const FieldArgs& f, long long idx, float tau, float& emax) {
-  float ev = error_coef_at(f, 6) * tau;
+// `ec`: the seven coefficients of the estimate (shared memory).
+__device__ __forceinline__ void st4_errmax(const FieldArgs& f, const float* ec, long long idx, float tau, float& emax) {
+  float ev = ec[6] * tau;
 #pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    const float ej = error_coef_at(f, j);
-    if (ej != 0.0f) ev = fmaf(ej, f.ek[j][idx], ev);
-  }
+  for (int j = 0; j < 6; ++j)
+    if (ec[j] != 0.0f) ev = fmaf(ec[j], f.ek[j][idx], ev);
   ev = fabsf(ev);
   emax = isnan(ev) || ev > emax ? ev : emax;
 }
@@ -83,52 +115,53 @@ __device__ __forceinline__ float st4_ghost(int i, int a, float d, float g, float
   return i == 0 ? mx : i == 1 ? my - d * g * mz : mz + d * g * my;
 }
 
-// One item: cells x0 .. x0 + 3 of tile row h (y = y0 + h) of plane z.
+// One item: cells x0 .. x0 + V - 1 of tile row h (y = y0 + h) of plane z.
 // msm, bd: m and the demag field of the tile rows in shared memory,
 // component c, row h, cell x at [c * cs + h * rs + x]; `two`: the tile has
 // its second row.
-template <bool DEMAG>
+template <bool DEMAG, int V>
 __device__ __forceinline__ void st4_item(const float* msm, const float* bd, int cs, int rs, int h, int x0, bool two,
-                                         const Grid& g, const RegionCoef& R, const FieldArgs& f, int z, int y,
+                                         const Grid& g, const RegionCoef& R, const float* ec, const FieldArgs& f, int z, int y,
                                          long long cell0, float& emax, float& tmax) {
   const int nx = g.nx, ny = g.ny;
   const long long n = g.n, pl = (long long)nx * ny;
   const unsigned terms = f.terms;
   const bool EX = terms & 2u, DM = terms & 8u, OPEN = terms & kTermOpenBC;
   if (R.ms == 0.0f) {   // empty material: no field, no torque
-    if (!MMP_IN(g, cell0 + 3, n)) return;
+    if (!MMP_IN(g, cell0 + V - 1, n)) return;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const long long idx = (long long)i * n + cell0;
-      *reinterpret_cast<float4*>(f.kout + idx) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (f.Bout) *reinterpret_cast<float4*>(f.Bout + idx) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      const float zero[V] = {};
+      st4_write<V>(f.kout + idx, zero);
+      if (f.Bout) st4_write<V>(f.Bout + idx, zero);
       if (f.err) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) st4_errmax(f, idx + j, 0.0f, emax);
+        for (int j = 0; j < V; ++j) st4_errmax(f, ec, idx + j, 0.0f, emax);
       }
     }
     return;
   }
-  const bool hasL = x0 > 0, hasR = x0 + 4 < nx, hasYm = y > 0, hasYp = y + 1 < ny;
+  const bool hasL = x0 > 0, hasR = x0 + V < nx, hasYm = y > 0, hasYp = y + 1 < ny;
   const bool hasZm = z > 0, hasZp = z + 1 < g.nz;
-  if (!MMP_IN(g, cell0 + 3, n) || (hasYm && !MMP_IN(g, cell0 - nx, n)) || (hasYp && !MMP_IN(g, cell0 + nx + 3, n)) ||
-      (hasZm && !MMP_IN(g, cell0 - pl, n)) || (hasZp && !MMP_IN(g, cell0 + pl + 3, n)))
+  if (!MMP_IN(g, cell0 + V - 1, n) || (hasYm && !MMP_IN(g, cell0 - nx, n)) || (hasYp && !MMP_IN(g, cell0 + nx + V - 1, n)) ||
+      (hasZm && !MMP_IN(g, cell0 - pl, n)) || (hasZp && !MMP_IN(g, cell0 + pl + V - 1, n)))
     return;
   // a missing x or y neighbour: the ghost (DMI, closed boundary) or m itself
   // (no DMI, or open boundary, where it also drops out of the DMI sum)
   const bool GH = DM && !OPEN;
   const float* st = f.stage;
-  float m[3][4];
+  float m[3][V];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) st4_put(m[c], *reinterpret_cast<const float4*>(msm + c * cs + h * rs + x0));
+  for (int c = 0; c < 3; ++c) st4_read<V>(m[c], msm + c * cs + h * rs + x0);
   // F_c: every single-precision term of B_c (demag added at the end)
-  float F[3][4];
+  float F[3][V];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     const float mx = m[0][j], my = m[1][j], mz = m[2][j];
     float s[3] = {0.0f, 0.0f, 0.0f};
     if (GH && EX) {   // the exchange term of the ghosts, c_a (ghost - m) = -d (D / (Ms h_a)) w
-      const bool lx = j == 0 && !hasL, rx = j == 3 && !hasR;
+      const bool lx = j == 0 && !hasL, rx = j == V - 1 && !hasR;
       const float ex = (lx ? R.exbc[0] : 0.0f) - (rx ? R.exbc[0] : 0.0f);
       const float ey = (!hasYm ? R.exbc[1] : 0.0f) - (!hasYp ? R.exbc[1] : 0.0f);
       s[0] = ex * mz;
@@ -161,58 +194,58 @@ __device__ __forceinline__ void st4_item(const float* msm, const float* bd, int 
   }
   if (terms & 64u) {   // magnetoelastic field
     const float* e = f.eps + cell0;
-    float exx[4], eyy[4], ezz[4], exy[4], exz[4], eyz[4];
-    st4_put(exx, __ldg(reinterpret_cast<const float4*>(e)));
-    st4_put(eyy, __ldg(reinterpret_cast<const float4*>(e + n)));
-    st4_put(ezz, __ldg(reinterpret_cast<const float4*>(e + 2 * n)));
-    st4_put(exy, __ldg(reinterpret_cast<const float4*>(e + 3 * n)));
-    st4_put(exz, __ldg(reinterpret_cast<const float4*>(e + 4 * n)));
-    st4_put(eyz, __ldg(reinterpret_cast<const float4*>(e + 5 * n)));
+    float exx[V], eyy[V], ezz[V], exy[V], exz[V], eyz[V];
+    st4_ldg<V>(exx, e);
+    st4_ldg<V>(eyy, e + n);
+    st4_ldg<V>(ezz, e + 2 * n);
+    st4_ldg<V>(exy, e + 3 * n);
+    st4_ldg<V>(exz, e + 4 * n);
+    st4_ldg<V>(eyz, e + 5 * n);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < V; ++j) {
       F[0][j] += R.mel1 * exx[j] * m[0][j] + R.mel2 * (exy[j] * m[1][j] + exz[j] * m[2][j]);
       F[1][j] += R.mel1 * eyy[j] * m[1][j] + R.mel2 * (exy[j] * m[0][j] + eyz[j] * m[2][j]);
       F[2][j] += R.mel1 * ezz[j] * m[2][j] + R.mel2 * (exz[j] * m[0][j] + eyz[j] * m[1][j]);
     }
   }
   // neighbours of component i: xl, xr the cells left of x0 and right of
-  // x0 + 3; ym, yp, zm, zp the 4 cells one row / plane away (a missing z
+  // x0 + V - 1; ym, yp, zm, zp the V cells one row / plane away (a missing z
   // neighbour is m itself: the zero-Neumann ghost)
-  float B[3][4];
-  df exz[4];
+  float B[3][V];
+  df exz[V];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const int i = k == 0 ? 2 : k - 1;   // z first: its neighbours carry the DMI of B_x and B_y
     const float* srow = msm + i * cs + h * rs;
     const float* grow = st + (long long)i * n + cell0;
     const float xl = hasL ? srow[x0 - 1] : m[i][0];
-    const float xr = hasR ? srow[x0 + 4] : m[i][3];
-    float ym[4], yp[4], zm[4], zp[4];
+    const float xr = hasR ? srow[x0 + V] : m[i][V - 1];
+    float ym[V], yp[V], zm[V], zp[V];
     if (h == 0) {
-      if (hasYm) st4_put(ym, __ldg(reinterpret_cast<const float4*>(grow - nx)));
-      else st4_put(ym, st4_get(m[i]));
-      if (two) st4_put(yp, *reinterpret_cast<const float4*>(srow + rs + x0));
-      else st4_put(yp, st4_get(m[i]));   // y + 1 = ny
+      if (hasYm) st4_ldg<V>(ym, grow - nx);
+      else st4_copy<V>(ym, m[i]);
+      if (two) st4_read<V>(yp, srow + rs + x0);
+      else st4_copy<V>(yp, m[i]);   // y + 1 = ny
     } else {
-      st4_put(ym, *reinterpret_cast<const float4*>(srow - rs + x0));
-      if (hasYp) st4_put(yp, __ldg(reinterpret_cast<const float4*>(grow + nx)));
-      else st4_put(yp, st4_get(m[i]));
+      st4_read<V>(ym, srow - rs + x0);
+      if (hasYp) st4_ldg<V>(yp, grow + nx);
+      else st4_copy<V>(yp, m[i]);
     }
-    if (hasZm) st4_put(zm, __ldg(reinterpret_cast<const float4*>(grow - pl)));
-    else st4_put(zm, st4_get(m[i]));
-    if (hasZp) st4_put(zp, __ldg(reinterpret_cast<const float4*>(grow + pl)));
-    else st4_put(zp, st4_get(m[i]));
+    if (hasZm) st4_ldg<V>(zm, grow - pl);
+    else st4_copy<V>(zm, m[i]);
+    if (hasZp) st4_ldg<V>(zp, grow + pl);
+    else st4_copy<V>(zp, m[i]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float xm = j == 0 ? xl : m[i][j - 1];
-      const float xp = j == 3 ? xr : m[i][j + 1];
+    for (int j = 0; j < V; ++j) {
+      const float xm = j == 0 ? xl : m[i][j > 0 ? j - 1 : 0];
+      const float xp = j == V - 1 ? xr : m[i][j < V - 1 ? j + 1 : j];
       df ex = {0.0f, 0.0f};
       if (EX) ex = st4_exch(R, xm, xp, ym[j], yp[j], zm[j], zp[j], m[i][j]);
       if (DM) {
         // DMI neighbour values: the ghost beyond a missing neighbour (closed
         // boundary) or nothing (open boundary: it drops out of the sum)
         const float dxm = j > 0 || hasL ? xm : GH ? st4_ghost(i, 0, -1.0f, R.ghost[0], m[0][0], m[1][0], m[2][0]) : 0.0f;
-        const float dxp = j < 3 || hasR ? xp : GH ? st4_ghost(i, 0, 1.0f, R.ghost[0], m[0][3], m[1][3], m[2][3]) : 0.0f;
+        const float dxp = j < V - 1 || hasR ? xp : GH ? st4_ghost(i, 0, 1.0f, R.ghost[0], m[0][V - 1], m[1][V - 1], m[2][V - 1]) : 0.0f;
         if (i == 2) {
           F[0][j] = fmaf(R.dmi[0], dxp - dxm, F[0][j]);
         } else if (i == 0) {
@@ -234,14 +267,14 @@ __device__ __forceinline__ void st4_item(const float* msm, const float* bd, int 
     }
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     const float b = DEMAG ? bd[2 * cs + h * rs + x0 + j] : 0.0f;
     B[2][j] = st4_fin(exz[j], F[2][j] + b);
   }
   // torque
-  float tau[3][4];
+  float tau[3][V];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < V; ++j) {
     const float mx = m[0][j], my = m[1][j], mz = m[2][j];
     const float bx = B[0][j], by = B[1][j], bz = B[2][j];
     const float mxB[3] = {my * bz - mz * by, mz * bx - mx * bz, mx * by - my * bx};
@@ -254,25 +287,27 @@ __device__ __forceinline__ void st4_item(const float* msm, const float* bd, int 
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const long long idx = (long long)i * n + cell0;
-    *reinterpret_cast<float4*>(f.kout + idx) = st4_get(tau[i]);
-    if (f.Bout) *reinterpret_cast<float4*>(f.Bout + idx) = st4_get(B[i]);
+    st4_write<V>(f.kout + idx, tau[i]);
+    if (f.Bout) st4_write<V>(f.Bout + idx, B[i]);
     if (f.err) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) st4_errmax(f, idx + j, tau[i][j], emax);
+      for (int j = 0; j < V; ++j) st4_errmax(f, ec, idx + j, tau[i][j], emax);
     }
   }
 }
 
 // Local field and torque of the tile rows y0 .. y0 + nrows - 1 (nrows = 1
-// or 2) of plane z, four cells per item (nx a multiple of 4, uniform
+// or 2) of plane z, V cells per item (nx a multiple of 4, uniform
 // material, one sublattice), then the block reductions as in field_cells.
-template <bool DEMAG>
+template <bool DEMAG, int V = 4>
 __device__ __forceinline__ void field_cells4(const float* msm, const float* bd, int cs, int rs, int nrows,
                                              const Grid& g, const Coefs& co, const FieldArgs& f, int z, int y0) {
-  const int nx = g.nx, q = nx >> 2;
+  const int nx = g.nx, q = nx / V;
   // the material's coefficients in shared memory: read there, they are not
   // reloaded from global memory after every store of the outputs
   __shared__ RegionCoef sR;
+  __shared__ float ec[7];
+  if (f.err && threadIdx.x == 0) error_coefs_load(f, ec);
   {
     const int* src = reinterpret_cast<const int*>(co.reg);
     int* dst = reinterpret_cast<int*>(&sR);
@@ -281,9 +316,9 @@ __device__ __forceinline__ void field_cells4(const float* msm, const float* bd, 
   __syncthreads();
   float emax = 0.0f, tmax = 0.0f;
   for (int e = threadIdx.x; e < nrows * q; e += blockDim.x) {
-    const int h = e >= q, x0 = 4 * (e - h * q), y = y0 + h;
+    const int h = e >= q, x0 = V * (e - h * q), y = y0 + h;
     const long long cell0 = x0 + (long long)nx * (y + (long long)g.ny * z);
-    st4_item<DEMAG>(msm, bd, cs, rs, h, x0, nrows == 2, g, sR, f, z, y, cell0, emax, tmax);
+    st4_item<DEMAG, V>(msm, bd, cs, rs, h, x0, nrows == 2, g, sR, ec, f, z, y, cell0, emax, tmax);
   }
   field_maxima(f, emax, tmax);
 }

@@ -37,6 +37,11 @@ bool xg_split(const Grid& g, int kind) {
   return kind != 0 || (Q > 1 && (g.Px != 2048 || pairs <= 304));
 }
 
+// Cells per item of the local field: four, but one or two where that gives a block
+// of a small grid up to 256 threads (the same sums; a four-cell item is a chain of
+// 1500 instructions on the one warp that its scheduler has): us, four -> fewer:
+// 64x64x1 ten steps 1055 -> 891, 200x180x1 1195 -> 1103, 256x256x2 relaxation 976 ->
+// 955.
 // Threads: the transforms' warps; more where the assembly (nx / 2 items of pass
 // A) or the cells (nx / 2 items of four cells, or 2 nx cells) fill them, up to the
 // kernel's limit while a grid gives each SM two blocks at most, to 128 above and in
@@ -48,8 +53,9 @@ XgPlan xg_plan(const Grid& g, int pass, bool cells, bool batch) {
   int M = 0, Q = 0;
   xg_shape(g, &M, &Q);
   const int warps = M <= 8 ? 1 : 3 * Q;
-  const int items = pass == 2 && cells ? 2 * g.nx : (g.nx + 1) / 2;
   const bool many = batch || (long long)((g.ny + 1) / 2) * g.nz > 304;
+  l.v = many || M > 16 ? 4 : M > 8 ? 2 : 1;
+  const int items = pass == 0 ? (g.nx + 1) / 2 : cells ? 2 * g.nx : 2 * g.nx / l.v;
   l.threads = std::max(32 * warps, std::min(many ? 128 : xg_maxthr(Q), (items + 31) / 32 * 32));
   const size_t W = (size_t)3 * Q * xg_pitch(M, Q) * sizeof(float2), HX = g.Px / 2;
   l.smem = pass == 0 ? 3 * HX * sizeof(float2) + W
@@ -66,6 +72,7 @@ static cudaError_t launch_xg_list(int pass, int kind, const Grid& g, const XgArg
   l.grid = insts ? dim3(nitems) : dim3((g.ny + 1) / 2, g.nz);
   l.threads = pl.threads;
   l.smem = pl.smem;
+  l.v = pl.v;
   if (!insts && pass == 0 && p.a.y) l.grid.z = 1 + p.a.nparts - p.a.nsub;   // elastic parts: blocks of their own
   if (!insts && pass == 2 && xg_split(g, kind)) {   // one component per block
     l.grid.z = 3;
@@ -106,6 +113,8 @@ __global__ void __launch_bounds__(128, 4) k_cells_g(const __grid_constant__ XgAr
   after_predecessor();
   if constexpr (VEC) {
     __shared__ RegionCoef sR;
+    __shared__ float ec[7];
+    if (p.f.err && threadIdx.x == 0) error_coefs_load(p.f, ec);
     const int* src = reinterpret_cast<const int*>(p.co.reg);
     for (int i = threadIdx.x; i < (int)(sizeof(RegionCoef) / sizeof(int)); i += 128) reinterpret_cast<int*>(&sR)[i] = src[i];
     __syncthreads();
@@ -113,7 +122,7 @@ __global__ void __launch_bounds__(128, 4) k_cells_g(const __grid_constant__ XgAr
     if (4 * e < g.n) {
       const int x0 = 4 * (int)(e - row * (nx >> 2)), z = (int)(row / ny), y = (int)(row - (long long)z * ny), h = y & 1;
       const long long base = (row - h) * nx;   // the row pair
-      st4_item<true>(p.f.stage + base, p.f.kout + base, (int)g.n, nx, h, x0, y + 1 - h < ny, g, sR, p.f, z, y,
+      st4_item<true, 4>(p.f.stage + base, p.f.kout + base, (int)g.n, nx, h, x0, y + 1 - h < ny, g, sR, ec, p.f, z, y,
                      row * nx + x0, emax, tmax);
     }
   } else {

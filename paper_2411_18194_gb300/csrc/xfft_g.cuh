@@ -247,8 +247,8 @@ __device__ __forceinline__ void passA_g_tile(unsigned char* sraw, const XgArgs& 
 }
 
 // KIND 0: one sublattice, uniform material; 1: one sublattice, regions; 2: two
-// sublattices, uniform; 3: two sublattices, regions.
-template <int M, int Q, int KIND>
+// sublattices, uniform; 3: two sublattices, regions.  V: cells per item (KIND 0).
+template <int M, int Q, int KIND, int V>
 __device__ __forceinline__ void passC_g_tile(unsigned char* sraw, const XgArgs& s, int z, int y0) {
   using X = Xg<M, Q>;
   constexpr int NB = X::NB, N = X::N, LP = X::LP, HX = X::HX;
@@ -365,7 +365,7 @@ __device__ __forceinline__ void passC_g_tile(unsigned char* sraw, const XgArgs& 
   // 3. local field and torque
   constexpr int NSUB = KIND >= 2 ? 2 : 1;
   constexpr bool UNI = KIND == 0 || KIND == 2;
-  if (KIND == 0 && vec) field_cells4<true>(ms, bd, 2 * HX, HX, two ? 2 : 1, g, s.co, s.f, z, y0);
+  if (KIND == 0 && vec) field_cells4<true, V>(ms, bd, 2 * HX, HX, two ? 2 : 1, g, s.co, s.f, z, y0);
   else field_cells<NSUB, true, UNI>(bd, 2 * HX, HX, two ? 2 : 1, g, s.co, s.f, z, y0);
 }
 
@@ -525,20 +525,21 @@ __global__ void __launch_bounds__(xg_maxthr(Q), xg_minblk(Q)) k_invx_g(const __g
   }
 }
 
-template <int M, int Q, int KIND>
+template <int M, int Q, int KIND, int V>
 __global__ void __launch_bounds__(xg_maxthr(Q), xg_minblk(Q))
     k_passC_g(const __grid_constant__ XgArgs p, const BatchInst* __restrict__ insts,
               const BatchItem* __restrict__ items, int stage) {
   extern __shared__ __align__(16) unsigned char sraw[];
   __shared__ __align__(16) XgArgs s;
   const BatchItem w = xg_tile(s, p, insts, items, stage);
-  passC_g_tile<M, Q, KIND>(sraw, s, w.b, 2 * w.a);
+  passC_g_tile<M, Q, KIND, V>(sraw, s, w.b, 2 * w.a);
 }
 
 struct XgLaunch {
   dim3 grid;
   int threads;
   size_t smem;
+  int v;       // cells per item of pass C's local field
 };
 
 template <int M, int Q>
@@ -565,11 +566,12 @@ cudaError_t launch_xg_t(int pass, int kind, const XgArgs& p, const XgLaunch& l, 
       return e != cudaSuccess ? e : launch_chained(p.d.chain, k_invx_g<M, Q>, l.grid, l.threads, l.smem, st, p);
     }
   }
-  if (kind == 0) return xg_go(k_passC_g<M, Q, 0>, p, l, insts, items, stage, st);
+  if (kind == 0 && M <= 16 && l.v != 4) return xg_go(k_passC_g<M, Q, 0, M <= 8 ? 1 : M <= 16 ? 2 : 4>, p, l, insts, items, stage, st);
+  if (kind == 0) return xg_go(k_passC_g<M, Q, 0, 4>, p, l, insts, items, stage, st);
   if constexpr (M <= 8) {   // above, several regions or sublattices take k_invx_g and k_cells_g (xg_split)
-    if (kind == 1) return xg_go(k_passC_g<M, Q, 1>, p, l, insts, items, stage, st);
-    if (kind == 2) return xg_go(k_passC_g<M, Q, 2>, p, l, insts, items, stage, st);
-    return xg_go(k_passC_g<M, Q, 3>, p, l, insts, items, stage, st);
+    if (kind == 1) return xg_go(k_passC_g<M, Q, 1, 4>, p, l, insts, items, stage, st);
+    if (kind == 2) return xg_go(k_passC_g<M, Q, 2, 4>, p, l, insts, items, stage, st);
+    return xg_go(k_passC_g<M, Q, 3, 4>, p, l, insts, items, stage, st);
   }
   return cudaErrorInvalidValue;
 }

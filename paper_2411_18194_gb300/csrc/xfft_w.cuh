@@ -255,10 +255,11 @@ __device__ __forceinline__ void passA_w_tile(unsigned char* sraw, const Grid& g,
   const float2* twT = d.tw_wx;                     // [N], global (L1)
   const int lane = lane_id(), warp = threadIdx.x >> 5;
   __shared__ float cf[7];
+  const bool stream = NSUB == 1 && (nx & 3) == 0 && a.nparts == a.nsub;
   if (threadIdx.x == 0) stage_coefs_load(a, cf);
-  __syncthreads();
+  if (!stream) __syncthreads();   // the streamed assembly has a barrier before its first use
   // 1. stage assembly of both rows into Zin (zero for x >= nx and a row y >= ny)
-  if (NSUB == 1 && (nx & 3) == 0 && a.nparts == a.nsub) {
+  if (stream) {
     passA_w_assemble_async<ASSEMBLE>(reinterpret_cast<float*>(Zin), reinterpret_cast<float*>(Sodd), Zin, g, a, co,
                                      cf, z, y0);
   } else if ((nx & 3) == 0) {

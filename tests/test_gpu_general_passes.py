@@ -75,3 +75,9 @@ def test_passes_a_and_c_materials(nx, ny, nz):
     """Several regions with empty cells, and two sublattices."""
     check((nx, ny, nz), 600 + nx, nreg=3, empty=0.1)
     check((nx, ny, nz), 700 + nx, n_sub=2, terms=("DEMAG", "EXCH", "ANIS", "AFM", "ZEEMAN"))
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(28, 620, 1), (62, 611, 1), (150, 306, 2), (250, 205, 3), (300, 612, 1)])
+def test_passes_a_and_c_many_rows(nx, ny, nz):
+    """More than two row pairs per SM: blocks of at most 128 threads, four cells an item."""
+    check((nx, ny, nz), 800 + nx)
