@@ -5,10 +5,10 @@
 // (member, tile) items of all active members: pass A (stage assembly +
 // forward x FFT) over their y tiles, pass B over their kx planes, pass C
 // (inverse x FFT + field + torque + error) over their tiles.  One block per
-// item.  A pass is one launch per (z-extent group for pass B, whose z
-// transform is specialised per nz; block-size class: each member's own block
-// size rounded up to 128, 256 or 512), and these launches run concurrently
-// on side streams, so small items run in small blocks several to an SM.
+// item.  A pass is one launch per padded length (the general warp kernels,
+// xfft_g.cuh and passb_g.cuh; pass B per nz too) and block size, or on the block
+// engine per z-extent group and block-size class, dealt over the batch stream and
+// two side streams, so small items run in small blocks several to an SM.
 // Each list is sorted by decreasing work, so uneven members share the GPU
 // without a tail per member.  Stream order makes pass B wait for pass A and
 // pass C for pass B.
@@ -250,6 +250,13 @@ BatchInst make_inst(const Member& m, unsigned* red, double h, int relax) {
   return I;
 }
 
+// Streams that the launches of one pass are dealt over.  One per launch (up to 13
+// in a mixed batch) interleaved the blocks of members that do not fit the L2 cache
+// together and paid an event pair each; with one, small launches leave SMs idle.
+// us at one per launch, 4, 3, 2, 1: batch of 24 31463, 28086, 29509, 30323, 38866; 8
+// relaxations 6000, 5921, 5577, 5449, 6395; 36 members 24092, 21423, 21293, 21681, -.
+constexpr size_t kPassStreams = 3;
+
 // Work lists over `mem` (member indices): per pass kind, z group (pass B)
 // and block-size class, one launch over its items sorted longest first;
 // uploaded to d_items.
@@ -349,7 +356,7 @@ int build_list(mmp_batch* b, const std::vector<int>& mem) {
     widest = std::max(widest, n);
   }
   if (!b->fork) BCK(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "batch: event");
-  while (b->aux.size() + 1 < widest) {
+  while (b->aux.size() + 1 < std::min(widest, kPassStreams)) {
     cudaStream_t st;
     cudaEvent_t ev;
     BCK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking), "batch: side stream");
@@ -406,16 +413,19 @@ int launch_stage(mmp_batch* b, int stage) {
       if (l.kind == kind) ls.push_back(&l);
     if (ls.empty()) continue;
     BTraced t(b, kind);
-    if (ls.size() > 1) BCK(cudaEventRecord(b->fork, b->stream), "batch: fork");
+    const size_t used = std::min(ls.size(), kPassStreams);
+    if (used > 1) {
+      BCK(cudaEventRecord(b->fork, b->stream), "batch: fork");
+      for (size_t i = 1; i < used; ++i) BCK(cudaStreamWaitEvent(b->aux[i - 1], b->fork, 0), "batch: fork wait");
+    }
     for (size_t i = 0; i < ls.size(); ++i) {
-      cudaStream_t s = i == 0 ? b->stream : b->aux[i - 1];
-      if (i > 0) BCK(cudaStreamWaitEvent(s, b->fork, 0), "batch: fork wait");
-      BCK(launch_one(b, *ls[i], stage, s), "batch: pass launch");
+      const size_t at = i % used;
+      BCK(launch_one(b, *ls[i], stage, at == 0 ? b->stream : b->aux[at - 1]), "batch: pass launch");
       b->launches++;
-      if (i > 0) {
-        BCK(cudaEventRecord(b->join[i - 1], s), "batch: join");
-        BCK(cudaStreamWaitEvent(b->stream, b->join[i - 1], 0), "batch: join wait");
-      }
+    }
+    for (size_t i = 1; i < used; ++i) {
+      BCK(cudaEventRecord(b->join[i - 1], b->aux[i - 1]), "batch: join");
+      BCK(cudaStreamWaitEvent(b->stream, b->join[i - 1], 0), "batch: join wait");
     }
   }
   return MMP_OK;
