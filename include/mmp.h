@@ -291,8 +291,11 @@ typedef struct mmp_shape {
     int stage_kernel;  /* 1: pass B stages its slice of the kernel octant in shared memory */
     int tyc;           /* rows per tile of pass C (inverse x FFT + field): 2, 4, 8, or 0 = the
                           default (ty, fewer when a block cannot hold its row pairs) */
-    int engine;        /* FFT engine, bit mask (0 = the block-wide Stockham passes, any
-                          supported grid):
+    int engine;        /* FFT engine, bit mask (0 = the general warp passes where they
+                          apply: passes A and C at padded x lengths of 64 and more, to
+                          which ty, tyc and radix_x then do not apply; pass B at R = 1,
+                          padded y lengths of 64 .. 2048 and nz <= 8, without radix_y
+                          and stage_kernel; the block-wide Stockham passes otherwise):
                           MMP_ENGINE_WARP_B: pass B on warp-level transforms (one warp
                           per column, in-register DFTs and one shared-memory transpose;
                           folded y length Py/R of 256, 512 or 1024, ny <= Py/R, R of 1

@@ -743,9 +743,9 @@ int replay_attempt(mmp_ctx* ctx, double h, int relax) {
       if (e == cudaSuccess) e = e2;
     }
     ctx->stream = user;
-    TRY(rc);
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&a->exec, gr, 0);
+    if (rc == MMP_OK && e == cudaSuccess) e = cudaGraphInstantiate(&a->exec, gr, 0);
     if (gr) cudaGraphDestroy(gr);
+    TRY(rc);
     CK(e, "capture attempt");
     a->y = ctx->d_y;
     a->k0 = ctx->d_k[0];

@@ -81,3 +81,21 @@ def test_passes_a_and_c_materials(nx, ny, nz):
 def test_passes_a_and_c_many_rows(nx, ny, nz):
     """More than two row pairs per SM: blocks of at most 128 threads, four cells an item."""
     check((nx, ny, nz), 800 + nx)
+
+
+@pytest.mark.parametrize("shape,cell", [
+    ((3, 2, 1), (2e-9, 2e-9, 2e-9)),        # fewer cells than lattice points: the differences point by point
+    ((12, 11, 3), (2e-9, 2e-9, 2e-9)),      # offsets on both sides of the cutoff along x and y
+    ((40, 9, 16), (4e-9, 4e-9, 5e-10)),     # every layer below the cutoff
+    ((70, 50, 2), (1e-9, 4e-9, 2e-9)),      # unequal cells
+    ((33, 200, 1), (2e-9, 3e-9, 2e-9)),     # lengths 96 and 512: a radix-3 pass, line counts that fill no block
+])
+def test_kernel_build(shape, cell):
+    """The near-field lattice and the line-pair transforms of the demag kernel, demag field alone."""
+    w = config_small(shape, cell, 900 + shape[0], terms=("DEMAG",))
+    p = w.problem
+    mag = make_magnet(p, w.m0)
+    Bg, _ = gpu_eval(mag, p)
+    Bo, _ = oracle_eval(p, w.m0)
+    assert np.all(np.abs(Bg[0] - Bo[0]) <= field_tolerance(p, Bo[0], 0)), np.abs(Bg[0] - Bo[0]).max()
+    mag.close()
