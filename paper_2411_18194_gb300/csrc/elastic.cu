@@ -87,7 +87,7 @@ static dim3 elastic_grid(const Grid& g) {
 // about 80 a cell): a cell whose rows are all in the 4th-order bulk takes a path
 // with no selection between them, so that they are in flight together; the
 // selection per term and the 64-bit divisions of the index took most of the time
-// before: 25 and 59 us per launch at 1024x256x1 with two sublattices (cold L2).
+// before: 1024x256x1 with two sublattices, cold L2: strain 25 -> 20 us, force 59 -> 38.
 // Antiferromagnet 1024x256x1, four steps (25 launches of each): 4506 -> 3994 us.
 // HZ: nz > 1.
 template <bool HZ>

@@ -19,6 +19,11 @@
 // store with few blocks in flight.  Here three warps (one for M <= 8, all three
 // components in its lanes) do a row pair's transforms with warp barriers only,
 // and the smallest tile, one row pair, gives the most blocks.
+// Cold L2, us per launch now, A and C: 64x64x1 6.6 and 7.7, 512x512x1 11 and 16.5,
+// 2048x128x1 31 and 10 + 10 (two kernels; 47 as one), 1024x256x1 of two sublattices
+// 23 and 8 + 21 (A 45 and C 100 on the kernels of xfft_w.cuh).  Before, whole passes:
+// 512x512x1 run 1577 -> 726 us, 2048x128x1 run 4094 -> 1865, with what follows 630 and
+// 1337.
 #pragma once
 #include "batch.h"
 #include "copy.cuh"
