@@ -78,16 +78,20 @@ struct mmp_ctx {
   // side stream of the elastic kernels (evaluate); events: after pass A, strain, force
   cudaStream_t estream = nullptr;
   cudaEvent_t eev[3] = {nullptr, nullptr, nullptr};
-  // adaptive attempts (replay_attempt), one graph per side of the buffer swap
+  // adaptive attempts (replay_attempt): one graph per torque (run, relax) and side
+  // of the buffer swap, with every state buffer it has baked in
   struct AttemptGraph {
     cudaGraphExec_t exec = nullptr;
     float* y = nullptr;
-    float* k0 = nullptr;
-    int method = -1, relax = 0;
-    long long gen = -1;
+    float* stage = nullptr;
+    float* k[7] = {};
+  };
+  struct AttemptGraphs {
+    AttemptGraph side[2];
+    int method = -1;
+    long long gen = -1;        // configuration (with method) that `seen` counts the attempts of
+    int seen = 0;
   } ag[2];
-  long long ag_gen = -1;       // configuration whose attempts ag_seen counts
-  int ag_seen = 0;
   bool ag_fresh = false;       // the graph stream follows the context's stream
   long long config_gen = 0, g_config_gen = -1;   // bumped by changes a graph would have baked in
   // tracing

@@ -700,12 +700,31 @@ int attempt_stages(mmp_ctx* ctx, double h, bool want_err, int relax, bool dev) {
   return MMP_OK;
 }
 
+// The attempt graphs of the present configuration and method: graphs of an
+// earlier one go, and its first attempts are counted anew.
+mmp_ctx::AttemptGraphs& attempt_graphs(mmp_ctx* ctx, int relax) {
+  mmp_ctx::AttemptGraphs& G = ctx->ag[relax ? 1 : 0];
+  if (G.gen != ctx->config_gen || G.method != ctx->method) {
+    for (auto& a : G.side) {
+      if (a.exec) cudaGraphExecDestroy(a.exec);
+      a = mmp_ctx::AttemptGraph();
+    }
+    G.gen = ctx->config_gen;
+    G.method = ctx->method;
+    G.seen = 0;
+  }
+  return G;
+}
+
 // An adaptive attempt as one graph launch: the coefficients of its step size
 // and the cleared maxima copied from pinned memory, the kernels, the maxima
 // read back.  Launched one by one, the 18 or more kernels of an attempt cost the
 // host about 4 us each, more than most of them run at 512x512x1 and below.  A
 // configuration's first attempts are launched directly: a graph costs about as
-// much to make as two of them.  One graph for each side of the y/stage swap.
+// much to make as two of them.  One graph for each side of the y/stage swap.  A
+// graph replays only on the buffers that it was captured with: steps of other
+// methods swap k_1 with other slots, so y and k_1 alone don't say which buffer
+// accept() will take as the next k_1.
 int replay_attempt(mmp_ctx* ctx, double h, int relax) {
   const Tableau& T = tableau(ctx->method);
   float* hc = reinterpret_cast<float*>(ctx->h_red + 2);
@@ -713,16 +732,11 @@ int replay_attempt(mmp_ctx* ctx, double h, int relax) {
   for (int i = 1; i <= T.S; ++i) stage_coefs(T, h, i, hc + kRedStage + 7 * (i - 1));
   error_coefs(T, h, hc + kRedError);
   TRY(graph_stream(ctx));
-  mmp_ctx::AttemptGraph* a = nullptr;
-  for (auto& c : ctx->ag)
-    if (c.exec && c.y == ctx->d_y && c.k0 == ctx->d_k[0] && c.method == ctx->method && c.relax == relax &&
-        c.gen == ctx->config_gen)
-      a = &c;
-  if (!a) {
-    a = &ctx->ag[0];
-    if (ctx->ag[0].exec && ctx->ag[0].gen == ctx->config_gen && ctx->ag[0].method == ctx->method &&
-        ctx->ag[0].relax == relax)
-      a = &ctx->ag[1];
+  mmp_ctx::AttemptGraphs& G = attempt_graphs(ctx, relax);
+  mmp_ctx::AttemptGraph* a = &G.side[G.side[0].exec && G.side[0].y != ctx->d_y];
+  bool same = a->exec && a->y == ctx->d_y && a->stage == ctx->d_stage;
+  for (int i = 0; i <= T.S; ++i) same = same && a->k[i] == ctx->d_k[i];
+  if (!same) {
     if (a->exec) cudaGraphExecDestroy(a->exec);
     a->exec = nullptr;
     cudaStream_t user = ctx->stream;
@@ -748,10 +762,8 @@ int replay_attempt(mmp_ctx* ctx, double h, int relax) {
     TRY(rc);
     CK(e, "capture attempt");
     a->y = ctx->d_y;
-    a->k0 = ctx->d_k[0];
-    a->method = ctx->method;
-    a->relax = relax;
-    a->gen = ctx->config_gen;
+    a->stage = ctx->d_stage;
+    for (int i = 0; i < 7; ++i) a->k[i] = ctx->d_k[i];
   }
   if (!ctx->ag_fresh) {   // after the work already queued on the context's stream
     CK(cudaEventRecord(ctx->gev[0], ctx->stream), "graph event");
@@ -770,12 +782,12 @@ int replay_attempt(mmp_ctx* ctx, double h, int relax) {
 // back (one synchronisation).
 int attempt(mmp_ctx* ctx, double h, bool want_err, int relax, double* err_out, double* tmax_out) {
   TRY(ensure_k1(ctx, relax));
-  if (ctx->ag_gen != ctx->config_gen) {
-    ctx->ag_gen = ctx->config_gen;
-    ctx->ag_seen = 0;
+  bool graph = false;
+  if (want_err) {
+    mmp_ctx::AttemptGraphs& G = attempt_graphs(ctx, relax);
+    graph = !ctx->prof && G.seen >= 4;
+    G.seen += G.seen < 4;
   }
-  const bool graph = want_err && !ctx->prof && ctx->ag_seen >= 4;
-  if (want_err) ctx->ag_seen += ctx->ag_seen < 4;
   if (graph) {
     TRY(replay_attempt(ctx, h, relax));
   } else {
@@ -1072,8 +1084,9 @@ int mmp_destroy(mmp_ctx* ctx) {
   if (ctx->estream) cudaStreamSynchronize(ctx->estream);
   release_khat(ctx);
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
-  for (auto& a : ctx->ag)
-    if (a.exec) cudaGraphExecDestroy(a.exec);
+  for (auto& G : ctx->ag)
+    for (auto& a : G.side)
+      if (a.exec) cudaGraphExecDestroy(a.exec);
   if (ctx->gstream) cudaStreamDestroy(ctx->gstream);
   for (cudaEvent_t ev : ctx->gev)
     if (ev) cudaEventDestroy(ev);

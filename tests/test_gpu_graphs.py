@@ -90,3 +90,34 @@ def test_batch_graph_and_split_pass_c_equal_solo():
             assert np.array_equal(_m(mag), m)
             assert [mag.time()[k] for k in ("t", "dt", "steps", "rejected")] == t
             mag.close()
+
+
+def test_adaptive_graph_after_steps_of_other_methods():
+    """Steps of methods with other stage counts swap k_1 with other buffers: after one fixed step each of
+    Heun, Bogacki-Shampine, Dormand-Prince and Heun, y and k_1 are where the attempt graphs were captured and
+    the buffer of the last stage is not."""
+    res = []
+    for traced in (False, True):
+        p, mag = _magnet((48, 40, 1), 21)
+        mag.set_solver(adaptive=True, dt=2e-14, tol=1e-5)
+        if traced:
+            mag.profile(True)
+        mag.step(8)          # both graphs captured
+        for method in ("HEUN", "BS23", "DP45", "HEUN"):
+            mag.set_solver(adaptive=False, dt=1e-14, method=method)
+            mag.step(1)
+        mag.set_solver(adaptive=True, dt=2e-14, tol=1e-5)
+        out = []
+        for _ in range(6):
+            mag.step(1)
+            t = mag.time()
+            out.append((_m(mag), t["t"], t["dt"], t["steps"], t["rejected"], t["evals"]))
+        mag.relax(torque_tol=1e-9, max_time=1.5e-13)   # the other torque, then the first one again
+        mag.step(7)
+        t = mag.time()
+        out.append((_m(mag), t["t"], t["dt"], t["steps"], t["rejected"], t["evals"]))
+        res.append(out)
+        mag.close()
+    for a, b in zip(*res):
+        assert np.array_equal(a[0], b[0])
+        assert a[1:] == b[1:]
