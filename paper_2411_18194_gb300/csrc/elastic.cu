@@ -75,12 +75,52 @@ __device__ __forceinline__ bool in_bulk(const int (&idx)[3], const int (&ext)[3]
   return b;
 }
 
-// Cells of row z ny + y by x: one thread a cell, rows over blockIdx.y (no
-// division by the extents).
+// Whether row idx of one axis of n cells is in the bulk of G (margin 2) or G^T (4).
+__device__ __forceinline__ bool axis_bulk(int idx, int n, int margin) { return idx >= margin && idx <= n - 1 - margin; }
+
+// One thread a cell, cells packed into blocks whatever the extents: a row of its own
+// blocks left most threads of a narrow grid idle, and a cell at one edge took the slow
+// rows along every axis (antiferromagnet without demag, us an evaluation, before ->
+// packed and by axis: 8x4096x1 151 -> 53, 129x8000x1 787 -> 298, 65x65x65 367 -> 150;
+// with demag 1024x1024x1 351 -> 293).  The coordinates come from exact divisions by
+// multiplication: 64-bit divisions cost the kernels a third of their time.
 constexpr int kElThreads = 128;
-static dim3 elastic_grid(const Grid& g) {
-  const long long rows = (long long)g.ny * g.nz;
-  return dim3((g.nx + kElThreads - 1) / kElThreads, (unsigned)(rows < 65535 ? rows : 65535));
+// q = c / d for 0 <= c < 2^31: m = ceil(2^(31 + l) / d), l = ceil(log2 d), so m < 2^32 and the
+// excess c (m d - 2^(31 + l)) / 2^(31 + l) stays below 1.
+struct FastDiv {
+  unsigned m, s, d;
+};
+static FastDiv fast_div(unsigned d) {
+  unsigned l = 0;
+  while ((1u << l) < d) ++l;
+  return {(unsigned)(((1ull << (31 + l)) + d - 1) / d), 31 + l, d};
+}
+__device__ __forceinline__ unsigned div_by(unsigned c, const FastDiv& f) {
+  return (unsigned)(((unsigned long long)c * f.m) >> f.s);
+}
+struct CellDiv {
+  FastDiv x, y;
+};
+static CellDiv cell_div(const Grid& g) { return {fast_div(g.nx), fast_div(g.ny)}; }
+template <bool HZ>
+__device__ __forceinline__ void cell_index(const CellDiv& f, unsigned cell, int (&idx)[3]) {
+  const unsigned row = div_by(cell, f.x), z = HZ ? div_by(row, f.y) : 0;
+  idx[0] = (int)(cell - row * f.x.d);
+  idx[1] = (int)(row - z * f.y.d);
+  idx[2] = (int)z;
+}
+
+// The three components' gradients along one axis (zero for one cell).
+__device__ __forceinline__ void grad3(const float* __restrict__ f, long long n, long long cell, int i, int ext,
+                                      long long st, float ih, float (&G)[3]) {
+  if (ext == 1) return;
+  if (axis_bulk(i, ext, 2)) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) G[j] = grad_bulk(f + j * n, cell, st, ih);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) G[j] = grad_at(f + j * n, cell, i, ext, st, ih);
+  }
 }
 
 // Both elastic kernels are bound by the latency of their neighbour loads (24 and
@@ -91,17 +131,16 @@ static dim3 elastic_grid(const Grid& g) {
 // Antiferromagnet 1024x256x1, four steps (25 launches of each): 4506 -> 3994 us.
 // HZ: nz > 1.
 template <bool HZ>
-__global__ void __launch_bounds__(kElThreads) k_strain(Grid g, ElasticArgs e, int nsub) {
+__global__ void __launch_bounds__(kElThreads) k_strain(Grid g, ElasticArgs e, CellDiv fd, int nsub) {
   const long long n = g.n;
   const float* u = e.stage + (long long)3 * nsub * n;
   const float* v = u + 3 * n;
-  const int x = blockIdx.x * kElThreads + threadIdx.x;
-  if (x >= g.nx) return;
   constexpr int NA = HZ ? 3 : 2;
-  for (int row = blockIdx.y; row < g.ny * g.nz; row += gridDim.y) {
-    const int z = HZ ? row / g.ny : 0, y = row - z * g.ny;
-    const long long cell = x + (long long)g.nx * row;
-    const int idx[3] = {x, y, z}, ext[3] = {g.nx, g.ny, g.nz};
+  const long long cell = (long long)blockIdx.x * kElThreads + threadIdx.x;
+  if (cell < n) {
+    int idx[3];
+    cell_index<HZ>(fd, (unsigned)cell, idx);
+    const int ext[3] = {g.nx, g.ny, g.nz};
     const long long st[3] = {1, g.nx, (long long)g.nx * g.ny};
     float G[3][3] = {}, Gv[3][3] = {};
     if (in_bulk(idx, ext, 2)) {
@@ -114,14 +153,12 @@ __global__ void __launch_bounds__(kElThreads) k_strain(Grid g, ElasticArgs e, in
 #pragma unroll
             for (int j = 0; j < 3; ++j) Gv[a][j] = grad_bulk(v + j * n, cell, st[a], g.ih[a]);
         }
-    } else {
+    } else {   // by axis: most of these cells are at the edge of one axis only
 #pragma unroll
-      for (int a = 0; a < NA; ++a)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          G[a][j] = grad_at(u + j * n, cell, idx[a], ext[a], st[a], g.ih[a]);
-          Gv[a][j] = e.eta != 0.0f ? grad_at(v + j * n, cell, idx[a], ext[a], st[a], g.ih[a]) : 0.0f;
-        }
+      for (int a = 0; a < NA; ++a) {
+        grad3(u, n, cell, idx[a], ext[a], st[a], g.ih[a], G[a]);
+        if (e.eta != 0.0f) grad3(v, n, cell, idx[a], ext[a], st[a], g.ih[a], Gv[a]);
+      }
     }
     float eps[6] = {G[0][0], G[1][1], G[2][2], 0.5f * (G[0][1] + G[1][0]), 0.5f * (G[0][2] + G[2][0]),
                     0.5f * (G[1][2] + G[2][1])};
@@ -149,7 +186,8 @@ __global__ void __launch_bounds__(kElThreads) k_strain(Grid g, ElasticArgs e, in
   }
 }
 
-// Force of one cell.  BULK: every row of G and G^T it needs is in the bulk.
+// Force of one cell.  BULK: every row of G and G^T it needs is in the bulk; else each
+// axis is looked at by itself.
 template <bool UNI, bool HZ, bool BULK>
 __device__ __forceinline__ void elastic_force(const Grid& g, const ElasticArgs& e, const Coefs& co, int nsub,
                                               long long cell, const int (&idx)[3], float (&f)[3]) {
@@ -160,11 +198,15 @@ __device__ __forceinline__ void elastic_force(const Grid& g, const ElasticArgs& 
   const long long st[3] = {1, g.nx, (long long)g.nx * g.ny};
 #pragma unroll
   for (int a = 0; a < NA; ++a)
-    if (!BULK || ext[a] > 1)
+    if (ext[a] > 1) {
+      if (BULK || axis_bulk(idx[a], ext[a], 4)) {
 #pragma unroll
-      for (int b = 0; b < 3; ++b)
-        f[b] -= BULK ? gradT_bulk(e.sig + sidx[a][b] * n, cell, st[a], g.ih[a])
-                     : gradT_at(e.sig + sidx[a][b] * n, cell, idx[a], ext[a], st[a], g.ih[a]);
+        for (int b = 0; b < 3; ++b) f[b] -= gradT_bulk(e.sig + sidx[a][b] * n, cell, st[a], g.ih[a]);
+      } else {
+#pragma unroll
+        for (int b = 0; b < 3; ++b) f[b] -= gradT_at(e.sig + sidx[a][b] * n, cell, idx[a], ext[a], st[a], g.ih[a]);
+      }
+    }
   if (!(e.terms & 64u)) return;
   const int reg = UNI ? 0 : co.regions[cell];
   for (int s = 0; s < nsub; ++s) {
@@ -172,12 +214,15 @@ __device__ __forceinline__ void elastic_force(const Grid& g, const ElasticArgs& 
     const RegionCoef& R = co.reg[s * MMP_MAX_REGIONS + reg];
     float G[3][3] = {};
 #pragma unroll
-    for (int a = 0; a < NA; ++a)
-      if (!BULK || ext[a] > 1)
+    for (int a = 0; a < NA; ++a) {
+      if (BULK) {
+        if (ext[a] > 1)
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
-          G[a][j] = BULK ? grad_bulk(m + j * n, cell, st[a], g.ih[a])
-                         : grad_at(m + j * n, cell, idx[a], ext[a], st[a], g.ih[a]);
+          for (int j = 0; j < 3; ++j) G[a][j] = grad_bulk(m + j * n, cell, st[a], g.ih[a]);
+      } else {
+        grad3(m, n, cell, idx[a], ext[a], st[a], g.ih[a], G[a]);
+      }
+    }
     const float mx = m[cell], my = m[n + cell], mz = m[2 * n + cell];
     const float B1 = R.b1, B2 = R.b2;
     f[0] += 2.0f * B1 * mx * G[0][0] + B2 * (mx * (G[1][1] + G[2][2]) + my * G[1][0] + mz * G[2][0]);
@@ -186,18 +231,20 @@ __device__ __forceinline__ void elastic_force(const Grid& g, const ElasticArgs& 
   }
 }
 
+// Six blocks an SM (72 registers): without the bound it takes 128 to 160 and the
+// 65x65x65 magnet 233 us an evaluation instead of 150, 1024x1024x1 320 instead of 293.
 template <bool UNI, bool HZ>
-__global__ void __launch_bounds__(kElThreads) k_elastic_rhs(Grid g, ElasticArgs e, Coefs co, int nsub) {
+__global__ void __launch_bounds__(kElThreads, 6) k_elastic_rhs(Grid g, ElasticArgs e, Coefs co, CellDiv fd,
+                                                            int nsub) {
   const long long n = g.n;
   const float* v = e.stage + (long long)3 * (nsub + 1) * n;
   float* ku = e.kout + (long long)3 * nsub * n;
   float* kv = ku + 3 * n;
-  const int x = blockIdx.x * kElThreads + threadIdx.x;
-  if (x >= g.nx) return;
-  for (int row = blockIdx.y; row < g.ny * g.nz; row += gridDim.y) {
-    const int z = HZ ? row / g.ny : 0, y = row - z * g.ny;
-    const long long cell = x + (long long)g.nx * row;
-    const int idx[3] = {x, y, z}, ext[3] = {g.nx, g.ny, g.nz};
+  const long long cell = (long long)blockIdx.x * kElThreads + threadIdx.x;
+  if (cell < n) {
+    int idx[3];
+    cell_index<HZ>(fd, (unsigned)cell, idx);
+    const int ext[3] = {g.nx, g.ny, g.nz};
     const float vc[3] = {v[cell], v[n + cell], v[2 * n + cell]};
     float f[3] = {0.0f, 0.0f, 0.0f};
     if (in_bulk(idx, ext, 4)) elastic_force<UNI, HZ, true>(g, e, co, nsub, cell, idx, f);
@@ -210,20 +257,24 @@ __global__ void __launch_bounds__(kElThreads) k_elastic_rhs(Grid g, ElasticArgs 
   }
 }
 
+static unsigned elastic_blocks(const Grid& g) { return (unsigned)((g.n + kElThreads - 1) / kElThreads); }
+
 cudaError_t launch_strain(const Grid& g, const ElasticArgs& e, int nsub, cudaStream_t s) {
-  if (g.nz > 1) k_strain<true><<<elastic_grid(g), kElThreads, 0, s>>>(g, e, nsub);
-  else k_strain<false><<<elastic_grid(g), kElThreads, 0, s>>>(g, e, nsub);
+  const CellDiv fd = cell_div(g);
+  if (g.nz > 1) k_strain<true><<<elastic_blocks(g), kElThreads, 0, s>>>(g, e, fd, nsub);
+  else k_strain<false><<<elastic_blocks(g), kElThreads, 0, s>>>(g, e, fd, nsub);
   return cudaGetLastError();
 }
 
 cudaError_t launch_elastic_rhs(const Grid& g, const ElasticArgs& e, const Coefs& c, int nsub, cudaStream_t s) {
-  const dim3 grid = elastic_grid(g);
+  const unsigned grid = elastic_blocks(g);
+  const CellDiv fd = cell_div(g);
   if (c.uniform) {
-    if (g.nz > 1) k_elastic_rhs<true, true><<<grid, kElThreads, 0, s>>>(g, e, c, nsub);
-    else k_elastic_rhs<true, false><<<grid, kElThreads, 0, s>>>(g, e, c, nsub);
+    if (g.nz > 1) k_elastic_rhs<true, true><<<grid, kElThreads, 0, s>>>(g, e, c, fd, nsub);
+    else k_elastic_rhs<true, false><<<grid, kElThreads, 0, s>>>(g, e, c, fd, nsub);
   } else {
-    if (g.nz > 1) k_elastic_rhs<false, true><<<grid, kElThreads, 0, s>>>(g, e, c, nsub);
-    else k_elastic_rhs<false, false><<<grid, kElThreads, 0, s>>>(g, e, c, nsub);
+    if (g.nz > 1) k_elastic_rhs<false, true><<<grid, kElThreads, 0, s>>>(g, e, c, fd, nsub);
+    else k_elastic_rhs<false, false><<<grid, kElThreads, 0, s>>>(g, e, c, fd, nsub);
   }
   return cudaGetLastError();
 }
