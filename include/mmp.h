@@ -396,6 +396,9 @@ int mmp_batch_advance(mmp_batch* b, int max_attempts, int* n_active);
 int mmp_batch_status(mmp_batch* b, mmp_ctx* ctx, int* done, int* status);
 /* Kernel launches the batch has made (tracing). */
 int mmp_batch_launches(mmp_batch* b, long long* n);
+/* Lock-step graphs the batch has made (tracing): one per set of active
+ * members and their shapes, kept between mmp_batch_advance calls. */
+int mmp_batch_graphs(mmp_batch* b, long long* n);
 /* Tracing: with enable != 0 (counters reset) every pass launch is bracketed
  * by CUDA events and fixed-step lock steps launch directly instead of
  * through the graph; mmp_batch_profile_read returns, for pass 0 (A: stage

@@ -94,6 +94,7 @@ _SIGS = {
     "mmp_batch_advance": ([_c.c_void_p, _c.c_int, _c.POINTER(_c.c_int)], _c.c_int),
     "mmp_batch_status": ([_c.c_void_p, _c.c_void_p, _c.POINTER(_c.c_int), _c.POINTER(_c.c_int)], _c.c_int),
     "mmp_batch_launches": ([_c.c_void_p, _c.POINTER(_c.c_longlong)], _c.c_int),
+    "mmp_batch_graphs": ([_c.c_void_p, _c.POINTER(_c.c_longlong)], _c.c_int),
     "mmp_batch_profile": ([_c.c_void_p, _c.c_int], _c.c_int),
     "mmp_batch_profile_read": ([_c.c_void_p, _c.c_int, _c.POINTER(_c.c_longlong), _c.POINTER(_c.c_double)],
                                _c.c_int),
@@ -470,6 +471,12 @@ class Batch:
     def launches(self):
         n = ctypes.c_longlong()
         _check(library().mmp_batch_launches(self._b, ctypes.byref(n)))
+        return n.value
+
+    def graphs(self):
+        """Lock-step graphs made so far."""
+        n = ctypes.c_longlong()
+        _check(library().mmp_batch_graphs(self._b, ctypes.byref(n)))
         return n.value
 
     def profile(self, enable=True):

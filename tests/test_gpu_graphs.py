@@ -121,3 +121,55 @@ def test_adaptive_graph_after_steps_of_other_methods():
     for a, b in zip(*res):
         assert np.array_equal(a[0], b[0])
         assert a[1:] == b[1:]
+
+
+def test_batch_keeps_its_graph_between_advances():
+    """Lock steps of one set of members replay one graph however the calls divide them; another set, or another
+    shape of a member between calls, makes a new one.  Bitwise the runs of the members alone."""
+    import paper_2411_18194_gb300 as pkg
+    shapes = [(64, 48, 1), (100, 60, 2), (40, 130, 1)]
+
+    def magnet(i):
+        p, mag = _magnet(shapes[i], 60 + i)
+        mag.set_shape(R=1, stage_kernel=0, engine=0)
+        mag.set_solver(adaptive=True, dt=2e-14, tol=1e-5)
+        return mag
+
+    mags, solo = ([magnet(i) for i in range(3)] for _ in range(2))
+    with pkg.Batch() as b:
+        for mag in mags:
+            b.add(mag, "steps", 24)
+        for _ in range(4):
+            assert b.advance(4) == 3
+        assert b.graphs() == 1
+        sh = mags[1].get_shape()
+        mags[1].set_shape(ty=4 if sh["ty"] == 2 else 2)
+        assert b.advance(4) == 3 and b.graphs() == 2
+        while b.advance(4):
+            pass
+        assert all(b.status(m) == (True, 0) for m in mags)
+    for i, (mag, s) in enumerate(zip(mags, solo)):
+        s.step(24)
+        t, ts = mag.time(), s.time()
+        if i != 1:   # member 1's change of shape drops its first stage: its own trajectory to rounding only
+            assert np.array_equal(_m(mag), _m(s))
+            assert [t[k] for k in ("t", "dt", "steps", "rejected")] == [ts[k] for k in ("t", "dt", "steps", "rejected")]
+        mag.close()
+        s.close()
+
+
+def test_batch_fixed_steps_keep_their_graph_between_advances():
+    import paper_2411_18194_gb300 as pkg
+    (p, mag), (_, solo) = _magnet((64, 48, 2), 71), _magnet((64, 48, 2), 71)
+    for x in (mag, solo):
+        x.set_shape(R=1, stage_kernel=0, engine=0)
+        x.set_solver(adaptive=False, dt=stable_dt(p))
+    with pkg.Batch() as b:
+        b.add(mag, "steps", 15)
+        while b.advance(4):
+            pass
+        assert b.graphs() == 1
+    solo.step(15)
+    assert np.array_equal(_m(mag), _m(solo))
+    for x in (mag, solo):
+        x.close()
