@@ -1,5 +1,10 @@
 // launch.cuh -- small host helpers shared by the launchers.
 #pragma once
+#include <algorithm>
+#include <map>
+#include <mutex>
+#include <utility>
+
 #include "kernels.h"
 
 namespace mmp {
@@ -9,10 +14,28 @@ static inline int grid_for(long long n, int threads) {
   return (int)(b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b));
 }
 
+inline cudaError_t raise_smem_limit(const void* kernel, size_t bytes) {
+  static std::mutex mu;
+  static std::map<std::pair<const void*, int>, size_t> limits;   // by kernel and device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  size_t& limit = limits[{kernel, dev}];
+  const size_t want = std::max(limit, bytes);
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+  if (e == cudaSuccess) limit = want;
+  return e;
+}
+
+// Dynamic shared memory above the default limit (fixed: the kernel's static shared
+// memory).  The limit belongs to the kernel, not to the launch: it only grows, or a
+// context on another host thread with a smaller need could lower it between this
+// call and the launch.
 template <typename K>
-static inline cudaError_t set_smem(K kernel, size_t bytes, size_t fixed = 0) {   // fixed: static shared memory
+static inline cudaError_t set_smem(K kernel, size_t bytes, size_t fixed = 0) {
   if (bytes + fixed <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return raise_smem_limit(reinterpret_cast<const void*>(kernel), bytes);
 }
 
 // A kernel that may be placed while its predecessor in the stream drains: its

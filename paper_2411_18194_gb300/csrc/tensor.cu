@@ -26,6 +26,7 @@
 //    line, shorter ones by the direct sums.
 #include <math.h>
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace mmp {
 
@@ -475,7 +476,7 @@ cudaError_t build_kernel_spectrum(const KernelBuild& kb, cudaStream_t s) {
     if (kb.P[a] >= 64) {   // FP64 FFT of line pairs
       const int np = fft64_pairs(kb.P[a]);
       const size_t sm = (size_t)2 * np * kb.P[a] * sizeof(double2);
-      cudaError_t err = cudaFuncSetAttribute(k_tensor_axis_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      const cudaError_t err = set_smem(k_tensor_axis_fft, sm);
       if (err != cudaSuccess) return err;
       const long long blocks = 6 * ((lines / 6 + 2 * np - 1) / (2 * np));
       k_tensor_axis_fft<<<(unsigned)blocks, kFft64Threads, sm, s>>>(src, dst, e[0], e[1], e[2], a, e[a], nout,
