@@ -122,8 +122,8 @@ struct FieldArgs {
   unsigned* torque_max;      // max |m x B| (float bits) in relax mode
 };
 
-// Coefficients of the stage (read once into shared memory: a selection at every
-// use between the stage loads kept them from being in flight together, and cost a
+// Coefficients of the stage (read once, into registers or shared memory: a selection at
+// every use between the stage loads kept them from being in flight together, and cost a
 // fifth of pass A) and coefficient j of the error estimate.
 __device__ __forceinline__ void stage_coefs_load(const StageArgs& a, float* cf) {
 #pragma unroll

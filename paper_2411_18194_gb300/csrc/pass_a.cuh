@@ -142,9 +142,10 @@ __device__ __forceinline__ void passA_tile(unsigned char* sraw, const Grid& g, c
   float2* tw = reinterpret_cast<float2*>(sraw + passa_twiddle_offset(Px, g.ty, g.xb));
   float* inv = reinterpret_cast<float*>(sraw + passa_inv_offset(Px, g.ty, g.xb));
   const long long n = g.n;
-  __shared__ float cf[7];
-  if (threadIdx.x == 0) stage_coefs_load(a, cf);
-  __syncthreads();
+  // coefficients in registers: from shared memory behind a barrier, 16x16x1 took 28.4 us an
+  // evaluation instead of 27.9, 16x2048x1 36.6 instead of 36.0
+  float cf[7];
+  if (ASSEMBLE) stage_coefs_load(a, cf);
   for (int i = threadIdx.x; i < Px; i += blockDim.x) tw[i] = __ldg(d.tw_x + i);
   if (ASSEMBLE && (a.normalize || a.nparts > a.nsub)) {
     for (int e = threadIdx.x; e < g.ty * nx; e += blockDim.x) {
