@@ -333,7 +333,8 @@ int mmp_set_shape(mmp_ctx* ctx, const mmp_shape* shape);
  * fastest: after a warm-up of ~100 ms of evaluations (loaded clocks), the
  * candidates of passes A+C (tile rows, x plan) and of pass B (R, staging,
  * y plan, block or warp engine) are timed separately in two interleaved rounds (CUDA events per
- * pass on the context's stream, the better round counts); the combination
+ * pass on the context's stream, the better round counts), one candidate for each set of kernels
+ * (shapes that differ in what their kernels don't use are one); the combination
  * replaces the starting shape only if a longer interleaved measurement
  * finds it > 2 % faster per evaluation.  Returns the shape (chosen, may be
  * NULL) and its time per field evaluation in ms (eval_ms, may be NULL).

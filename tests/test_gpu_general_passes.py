@@ -99,3 +99,19 @@ def test_kernel_build(shape, cell):
     Bo, _ = oracle_eval(p, w.m0)
     assert np.all(np.abs(Bg[0] - Bo[0]) <= field_tolerance(p, Bo[0], 0)), np.abs(Bg[0] - Bo[0]).max()
     mag.close()
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_autotune_times_each_set_of_kernels_once(batch):
+    """96 x 64 x 2 runs the general passes: one candidate of passes A and C, and of pass B the general kernel and
+    (not in a batch) four block shapes for each of R = 2, 4 and 8.  Five evaluations a candidate and round, 36 for
+    the final comparison, after a warm-up of 200 times five."""
+    w = config_small((96, 64, 2), (2e-9, 2e-9, 2e-9), 31, terms=("DEMAG", "EXCH"))
+    mag = make_magnet(w.problem, w.m0)
+    start = mag.get_shape()
+    before = mag.time()["evals"]
+    shape, _ = mag.autotune(batch=batch, force=True)
+    if not batch:
+        assert [shape[k] for k in ("ty", "tyc", "radix_x")] == [start[k] for k in ("ty", "tyc", "radix_x")]
+    assert mag.time()["evals"] - before <= 1000 + 2 * 5 * (2 if batch else 1 + 13) + 36
+    mag.close()
