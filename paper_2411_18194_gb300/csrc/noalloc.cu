@@ -43,9 +43,9 @@ struct Setup {
   bool ready = false;              // tables built for the geometry below
   int n[3] = {0, 0, 0};
   double cell[3] = {0, 0, 0};
-  Grid g;
-  DemagArgs d;
-  Coefs co;
+  Grid g{};
+  DemagArgs d{};
+  Coefs co{};
   float* tau = nullptr;
   int thrA = 0, thrB = 0, thrC = 0;
 };
@@ -93,7 +93,7 @@ int cuda_err(cudaError_t e, const char* what) {
 // Build the tables of one geometry into the scratch of the current device
 // (host-to-device copies, the FP64 kernel build, one synchronisation).
 int set_up(Setup& S, int nx, int ny, int nz, const double* cell, cudaStream_t s) {
-  Grid g;
+  Grid g{};   // no index checks in the bounds-checked build: there is no flag word to report in
   g.nx = nx; g.ny = ny; g.nz = nz;
   g.n = (long long)nx * ny * nz;
   g.Px = nice_length(nx); g.Py = nice_length(ny); g.Pz = nice_length(nz);
