@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kXwThreads, 4) k_batch_passA_w(const BatchInst
   __shared__ StageArgs sa;
   __shared__ FieldArgs fa;
   batch_member(insts, inst, stage, si, sa, fa);
-  passA_w_tile<1, ASSEMBLE>(sraw, si.g, sa, si.d, si.co, blockIdx.y, 2 * blockIdx.x);
+  passA_w_tile<ASSEMBLE>(sraw, si.g, sa, si.d, si.co, blockIdx.y, 2 * blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kXwThreads, 4) k_batch_field_w(const BatchInst* __restrict__ insts, int inst,
@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(kXwThreads, 4) k_batch_field_w(const BatchInst
   __shared__ StageArgs sa;
   __shared__ FieldArgs fa;
   batch_member(insts, inst, stage, si, sa, fa);
-  field_w_tile<1, true>(sraw, si.g, si.d, si.co, fa, blockIdx.y, 2 * blockIdx.x);
+  field_w_tile(sraw, si.g, si.d, si.co, fa, blockIdx.y, 2 * blockIdx.x);
 }
 
 template <int NZ>

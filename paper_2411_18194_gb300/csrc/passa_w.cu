@@ -1,10 +1,17 @@
 // passa_w.cu -- pass A on the warp FFT engine (body in xfft_w.cuh): kernel
-// instantiations and launcher.
+// and launcher.
 #include "kernels.h"
 #include "launch.cuh"
 #include "xfft_w.cuh"
 
 namespace mmp {
+
+template <bool ASSEMBLE>
+__global__ void __launch_bounds__(kXwThreads, 4) k_passA_w(Grid g, StageArgs a, DemagArgs d, Coefs co) {
+  extern __shared__ __align__(16) unsigned char sraw[];
+  after_predecessor();
+  passA_w_tile<ASSEMBLE>(sraw, g, a, d, co, blockIdx.y, 2 * blockIdx.x);
+}
 
 cudaError_t launch_passA_w(const Grid& g, const StageArgs& a, const DemagArgs& d, const Coefs& c, cudaStream_t s) {
   // two sublattices: the general pass, whose loads of a stage's vectors are in
@@ -17,7 +24,7 @@ cudaError_t launch_passA_w(const Grid& g, const StageArgs& a, const DemagArgs& d
     const cudaError_t e = set_smem(kernel, sm, 64);
     return e != cudaSuccess ? e : launch_chained(d.chain, kernel, grid, kXwThreads, sm, s, g, a, d, c);
   };
-  return a.stage != nullptr && a.y != nullptr ? go(k_passA_w<1, true>) : go(k_passA_w<1, false>);
+  return a.stage != nullptr && a.y != nullptr ? go(k_passA_w<true>) : go(k_passA_w<false>);
 }
 
 }  // namespace mmp

@@ -12,16 +12,16 @@
 //   A[k] = (Z[k] + conj Z[2N - k]) / 2,  B[k] = -i (Z[k] - conj Z[2N - k]) / 2,
 // where Z[2N - k] has the parity of k, so each warp pairs its own outputs.
 //
-// Pass A: stage assembly (16-byte loads of 4 cells), M = sum_s Ms m_s into
-// shared memory, forward transforms, the half spectra of both rows to T.
+// One sublattice (two take the passes of xfft_g.cuh), and in pass C one region.
+// Pass A: stage assembly (16-byte loads of 4 cells), M = Ms m into shared
+// memory, forward transforms, the half spectra of both rows to T.
 // Pass C: the half spectra of both rows gathered into shared memory with
 // asynchronous copies, inverse transforms, the demag field of the two rows,
 // then the local field and torque of every cell: four cells per item with
 // the tile rows of m staged in shared memory (stencil4.cuh), or one cell
-// per thread (field_cells) for two sublattices or several regions.
+// per thread (field_cells) where nx is not a multiple of 4.
 #pragma once
 #include "kernels.h"
-#include "launch.cuh"
 #include "wfft.cuh"
 #include "copy.cuh"
 #include "stage.cuh"
@@ -68,54 +68,47 @@ __device__ __forceinline__ float4 stage_value4(const Grid& g, const StageArgs& a
 
 // Assembly of one row (y) of the tile: cells x0 .. x0 + V - 1 (V = 4 with
 // 16-byte loads when nx is a multiple of 4, else V = 1), all parts, the
-// stage state written once, M_c = sum_s Ms m_s into Zin[c][x].h.
-template <int NSUB, bool ASSEMBLE, int V>
+// stage state written once, M_c = Ms m into Zin[c][x].h.
+template <bool ASSEMBLE, int V>
 __device__ __forceinline__ void passA_w_cells(const Grid& g, const StageArgs& a, const Coefs& co,
                                               const float* cf, float2* Zin, int h, int x0, long long cell0) {
   const long long n = g.n;
-  float Mv[3][V];
+  float m[3][V];
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int i = 0; i < V; ++i) Mv[c][i] = 0.0f;
-#pragma unroll
-  for (int s = 0; s < NSUB; ++s) {
-    float m[3][V];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if constexpr (V == 4) {
-        const float4 q = stage_value4<ASSEMBLE>(g, a, cf, n, s, c, cell0);
-        m[c][0] = q.x; m[c][1] = q.y; m[c][2] = q.z; m[c][3] = q.w;
-      } else {
-        m[c][0] = stage_value<ASSEMBLE>(g, a, cf, n, s, c, cell0);
-      }
+  for (int c = 0; c < 3; ++c) {
+    if constexpr (V == 4) {
+      const float4 q = stage_value4<ASSEMBLE>(g, a, cf, n, 0, c, cell0);
+      m[c][0] = q.x; m[c][1] = q.y; m[c][2] = q.z; m[c][3] = q.w;
+    } else {
+      m[c][0] = stage_value<ASSEMBLE>(g, a, cf, n, 0, c, cell0);
     }
-    if (ASSEMBLE && a.normalize) {
-#pragma unroll
-      for (int i = 0; i < V; ++i) {
-        const float nn = m[0][i] * m[0][i] + m[1][i] * m[1][i] + m[2][i] * m[2][i];
-        const float r = nn > 0.0f ? rnorm3df(m[0][i], m[1][i], m[2][i]) : 1.0f;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) m[c][i] *= r;
-      }
-    }
-    if (ASSEMBLE) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const long long idx = (long long)(3 * s + c) * n + cell0;
-        if (!MMP_IN(g, idx + V - 1, g.lim_state)) continue;
-        float* dst = a.stage + idx;
-        if constexpr (V == 4) *reinterpret_cast<float4*>(dst) = make_float4(m[c][0], m[c][1], m[c][2], m[c][3]);
-        else dst[0] = m[c][0];
-      }
-    }
+  }
+  if (ASSEMBLE && a.normalize) {
 #pragma unroll
     for (int i = 0; i < V; ++i) {
-      const int reg = co.uniform ? 0 : co.regions[cell0 + i];
-      const float ms = co.reg[s * MMP_MAX_REGIONS + reg].ms;
+      const float nn = m[0][i] * m[0][i] + m[1][i] * m[1][i] + m[2][i] * m[2][i];
+      const float r = nn > 0.0f ? rnorm3df(m[0][i], m[1][i], m[2][i]) : 1.0f;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) Mv[c][i] = fmaf(ms, m[c][i], Mv[c][i]);
+      for (int c = 0; c < 3; ++c) m[c][i] *= r;
     }
+  }
+  if (ASSEMBLE) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const long long idx = c * n + cell0;
+      if (!MMP_IN(g, idx + V - 1, g.lim_state)) continue;
+      float* dst = a.stage + idx;
+      if constexpr (V == 4) *reinterpret_cast<float4*>(dst) = make_float4(m[c][0], m[c][1], m[c][2], m[c][3]);
+      else dst[0] = m[c][0];
+    }
+  }
+  float Mv[3][V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) {
+    const int reg = co.uniform ? 0 : co.regions[cell0 + i];
+    const float ms = co.reg[reg].ms;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Mv[c][i] = fmaf(ms, m[c][i], 0.0f);
   }
   // elastic parts (u, v): assembled here, not transformed
   if (ASSEMBLE) {
@@ -245,7 +238,7 @@ __device__ __forceinline__ void passA_w_assemble_async(float* buf0, float* buf1,
   }
 }
 
-template <int NSUB, bool ASSEMBLE>
+template <bool ASSEMBLE>
 __device__ __forceinline__ void passA_w_tile(unsigned char* sraw, const Grid& g, const StageArgs& a,
                                              const DemagArgs& d, const Coefs& co, int z, int y0) {
   constexpr int N = kXwN;
@@ -255,7 +248,7 @@ __device__ __forceinline__ void passA_w_tile(unsigned char* sraw, const Grid& g,
   const float2* twT = d.tw_wx;                     // [N], global (L1)
   const int lane = lane_id(), warp = threadIdx.x >> 5;
   __shared__ float cf[7];
-  const bool stream = NSUB == 1 && (nx & 3) == 0 && a.nparts == a.nsub;
+  const bool stream = (nx & 3) == 0 && a.nparts == a.nsub;
   if (threadIdx.x == 0) stage_coefs_load(a, cf);
   if (!stream) __syncthreads();   // the streamed assembly has a barrier before its first use
   // 1. stage assembly of both rows into Zin (zero for x >= nx and a row y >= ny)
@@ -267,7 +260,7 @@ __device__ __forceinline__ void passA_w_tile(unsigned char* sraw, const Grid& g,
     for (int e = threadIdx.x; e < 2 * q; e += kXwThreads) {
       const int h = e >= q, x0 = 4 * (e - h * q), y = y0 + h;
       if (y < ny) {
-        passA_w_cells<NSUB, ASSEMBLE, 4>(g, a, co, cf, Zin, h, x0, x0 + (long long)nx * (y + (long long)ny * z));
+        passA_w_cells<ASSEMBLE, 4>(g, a, co, cf, Zin, h, x0, x0 + (long long)nx * (y + (long long)ny * z));
       } else {
         float* Zf = reinterpret_cast<float*>(Zin);
         for (int c = 0; c < 3; ++c)
@@ -278,7 +271,7 @@ __device__ __forceinline__ void passA_w_tile(unsigned char* sraw, const Grid& g,
     for (int e = threadIdx.x; e < 2 * nx; e += kXwThreads) {
       const int h = e >= nx, x0 = e - h * nx, y = y0 + h;
       if (y < ny) {
-        passA_w_cells<NSUB, ASSEMBLE, 1>(g, a, co, cf, Zin, h, x0, x0 + (long long)nx * (y + (long long)ny * z));
+        passA_w_cells<ASSEMBLE, 1>(g, a, co, cf, Zin, h, x0, x0 + (long long)nx * (y + (long long)ny * z));
       } else {
         float* Zf = reinterpret_cast<float*>(Zin);
         for (int c = 0; c < 3; ++c) Zf[2 * (c * N + x0) + h] = 0.0f;
@@ -329,7 +322,6 @@ __device__ __forceinline__ void passA_w_tile(unsigned char* sraw, const Grid& g,
 }
 
 // ------------------------------------------------------------- pass C ----
-template <int NSUB, bool UNI>
 __device__ __forceinline__ void field_w_tile(unsigned char* sraw, const Grid& g, const DemagArgs& d,
                                              const Coefs& co, const FieldArgs& f, int z, int y0) {
   constexpr int N = kXwN;
@@ -397,11 +389,10 @@ __device__ __forceinline__ void field_w_tile(unsigned char* sraw, const Grid& g,
     }
   }
   __syncthreads();
-  // 3. local field and torque of the two rows.  One sublattice of uniform
-  // material with nx a multiple of 4: the tile rows of m into the odd
-  // warps' scratch (free now; component c at floats 4 c N + 2 N) by 16-byte
+  // 3. local field and torque of the two rows.  nx a multiple of 4: the tile
+  // rows of m into the odd warps' scratch (free now; component c at floats 4 c N + 2 N) by 16-byte
   // asynchronous copies, then four cells per item (stencil4.cuh).
-  if (NSUB == 1 && UNI && (g.nx & 3) == 0) {
+  if ((g.nx & 3) == 0) {
     float* Sf = reinterpret_cast<float*>(S);
     const int nx = g.nx, q = nx >> 2, nrows = two ? 2 : 1;
     const long long n = g.n, row0 = (long long)nx * (y0 + (long long)ny * z);
@@ -415,23 +406,8 @@ __device__ __forceinline__ void field_w_tile(unsigned char* sraw, const Grid& g,
     __syncthreads();
     field_cells4<true>(Sf + 2 * N, Sf, 4 * N, N, nrows, g, co, f, z, y0);
   } else {
-    field_cells<NSUB, true, UNI>(reinterpret_cast<const float*>(S), 4 * N, N, 2, g, co, f, z, y0);
+    field_cells<1, true, true>(reinterpret_cast<const float*>(S), 4 * N, N, 2, g, co, f, z, y0);
   }
-}
-
-// ------------------------------------------------------------ kernels ----
-template <int NSUB, bool ASSEMBLE>
-__global__ void __launch_bounds__(kXwThreads, 4) k_passA_w(Grid g, StageArgs a, DemagArgs d, Coefs co) {
-  extern __shared__ __align__(16) unsigned char sraw[];
-  after_predecessor();
-  passA_w_tile<NSUB, ASSEMBLE>(sraw, g, a, d, co, blockIdx.y, 2 * blockIdx.x);
-}
-
-template <int NSUB, bool UNI>
-__global__ void __launch_bounds__(kXwThreads, 4) k_field_w(Grid g, DemagArgs d, Coefs co, FieldArgs f) {
-  extern __shared__ __align__(16) unsigned char sraw[];
-  after_predecessor();
-  field_w_tile<NSUB, UNI>(sraw, g, d, co, f, blockIdx.y, 2 * blockIdx.x);
 }
 
 }  // namespace mmp
