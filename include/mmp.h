@@ -347,14 +347,16 @@ int mmp_autotune(mmp_ctx* ctx, int flags, mmp_shape* chosen, double* eval_ms);
  * Batches: independent contexts advanced together (no counterpart in the
  * paper, which runs one simulation at a time).  In every Dormand-Prince
  * stage each of the three demag passes of all active members is launched
- * once per (z group, block-size class) over a work list of (member, tile)
- * items, one block per item, longest first; the launches of a pass run
- * concurrently on side streams and stream order carries the dependencies
- * between passes (there is no device-side wait).  Lock steps of
- * fixed-step members are replayed from a CUDA graph.  A member runs
- * exactly the arithmetic of its own context
- * (same plans and coefficients), so its results are bitwise those of
- * mmp_step / mmp_run / mmp_relax on the same context with the same shape.
+ * once per padded length (pass B: and nz) and block size over a work list of
+ * (member, tile) items, one block per item, longest first (members on the
+ * block passes: once per z group and block-size class); the launches of a
+ * pass run concurrently on side streams and stream order carries the
+ * dependencies between passes (there is no device-side wait).  Lock steps are
+ * replayed from a CUDA graph, those with errors read back from the third of
+ * one set of members on; graph and work list stay between mmp_batch_advance
+ * calls.  A member runs exactly the arithmetic of its own context (same plans
+ * and coefficients), so its results are bitwise those of mmp_step / mmp_run /
+ * mmp_relax on the same context with the same shape.
  *
  * Members: one sublattice, one region (no region map), the demag term on,
  * no AFM / magnetoelastic / elastic terms, and either the shape R = 1,

@@ -1,5 +1,5 @@
 // batch.cu -- many independent contexts advanced in lock step (host
-// driver; kernels in batch_a.cu, batch_b.cu, batch_c.cu).
+// driver; kernels in xfft_g.cuh, passb_g.cuh, batch_a.cu, batch_b.cu, batch_c.cu).
 //
 // Every pass of every Dormand-Prince stage runs over a work list of
 // (member, tile) items of all active members: pass A (stage assembly +
@@ -7,18 +7,19 @@
 // (inverse x FFT + field + torque + error) over their tiles.  One block per
 // item.  A pass is one launch per padded length (the general warp kernels,
 // xfft_g.cuh and passb_g.cuh; pass B per nz too) and block size, or on the block
-// engine per z-extent group and block-size class, dealt over the batch stream and
+// passes per z-extent group and block-size class, dealt over the batch stream and
 // two side streams, so small items run in small blocks several to an SM.
 // Each list is sorted by decreasing work, so uneven members share the GPU
 // without a tail per member.  Stream order makes pass B wait for pass A and
 // pass C for pass B.
-// A fixed-step lock step (6 stages and the accept) is one CUDA graph,
-// replayed.
+// A lock step is one CUDA graph, replayed: with fixed steps the 6 stages and the
+// accept; with errors read back the 6 stages, from the third lock step of one set
+// of members on.  List and graph stay between advance calls.
 //
 // Each member runs exactly the arithmetic of its own context path (the same
 // device bodies, FFT plans and FP32 stage coefficients formed from the same
 // FP64 step), so a member's trajectory is bitwise the same alone and in any
-// batch.  The batched pass B is one CTA per kx plane (R = 1) reading the
+// batch.  The batched pass B takes a kx plane in one CTA (R = 1) and reads the
 // kernel rows from L2; members must use that shape (mmp_set_shape, or
 // mmp_autotune with MMP_TUNE_BATCH).
 #include <math.h>
@@ -259,9 +260,8 @@ BatchInst make_inst(const Member& m, unsigned* red, double h, int relax) {
 // relaxations 6000, 5921, 5577, 5449, 6395; 36 members 24092, 21423, 21293, 21681, -.
 constexpr size_t kPassStreams = 3;
 
-// Work lists over `mem` (member indices): per pass kind, z group (pass B)
-// and block-size class, one launch over its items sorted longest first;
-// uploaded to d_items.
+// Work lists over `mem` (member indices): the launches of every pass, each over its
+// items sorted longest first; uploaded to d_items.
 int build_list(mmp_batch* b, const std::vector<int>& mem) {
   ListSet L;
   L.members = mem;

@@ -1,7 +1,7 @@
 // batch.h -- device side of the batched driver (batch.cu): the per-member
-// descriptor, work items, and the pass kernels over a work list, one block
-// per (member, tile) item, launched once per pass, z group and block-size
-// class (batch_a.cu, batch_b.cu, batch_c.cu).
+// descriptor, work items, and the block passes over a work list, one block
+// per (member, tile) item (batch_a.cu, batch_b.cu, batch_c.cu; the general warp
+// passes, which most members run, take the same items: xfft_g.cuh, passb_g.cuh).
 #pragma once
 #include "kernels.h"
 

@@ -45,8 +45,8 @@ struct mmp_ctx {
   float* d_khat = nullptr;     // shared spectrum (build_khat), not owned
   std::tuple<int, int, int, int, double, double, double> khat_key;
   float2 *d_tw_x = nullptr, *d_tw_y = nullptr, *d_tw_ly = nullptr, *d_tw_z = nullptr;
-  float2* d_tw_wy = nullptr;   // warp pass B twiddles (engine & MMP_ENGINE_WARP_B)
-  float2 *d_tw_wx = nullptr, *d_tw_wx2 = nullptr;   // warp passes A and C (MMP_ENGINE_WARP_X)
+  float2* d_tw_wy = nullptr;   // warp and general pass B twiddles (kernels.h)
+  float2 *d_tw_wx = nullptr, *d_tw_wx2 = nullptr;   // warp and general passes A and C (kernels.h)
   float* d_tw_tc = nullptr;    // tensor-core DFT32 matrices (MMP_ENGINE_TC_Y)
   unsigned* d_flag = nullptr;  // set by a device wait that ran past its limit
   unsigned* d_red = nullptr;   // [0] error bits, [1] torque bits, then the coefficients of an attempt

@@ -84,10 +84,10 @@ struct DemagArgs {
   FftPlan plan_x, plan_ly;
   int R;                     // residue classes of ky per cluster
   int ks;                    // pass B stages the kernel slice in shared memory
-  // warp engine (wfft.cuh): twiddle tables w_N^(l k1) at [k1 * 32 + l]
-  const float2* tw_wy;       // N = Ly (pass B; the general pass B: Py / Q)
-  const float2* tw_wx;       // N = Px / 2 (passes A and C)
-  const float2* tw_wx2;      // w_Px^x, x < Px / 2 (natural order; passes A and C)
+  // warp transforms (wfft.cuh, gfft.cuh): twiddle tables w_N^(l k1) at [k1 * 32 + l]
+  const float2* tw_wy;       // N = Ly (warp pass B) or Py / Q (general pass B)
+  const float2* tw_wx;       // N = Px / Q, Q classes of kx (passes A and C; Q = 2 in xfft_w.cuh)
+  const float2* tw_wx2;      // w_Px^x, x < Px (natural order; read at r x, class r < Q)
   const float* tw_tc;        // tensor-core DFT32 matrices, split TF32 (tcdft.cuh layout)
   unsigned* err;             // set to 1 by a device wait that ran past its limit
   int chain;                 // launch_chained for the warp passes (0 in captured graphs, see launch.cuh)
@@ -239,6 +239,9 @@ __host__ __device__ constexpr int xg_maxthr(int Q) { return Q == 4 ? 384 : 256; 
 // four steps 2780 -> 2972 us (pass A at 80) -> 3124 (both), 1024x256x1
 // antiferromagnet 2665 -> 2873.
 __host__ __device__ constexpr int xg_minblk(int Q) { return Q == 4 ? 1 : 2; }
+// Blocks of two a streaming multiprocessor (152): the line between grids that leave
+// the chip room and grids that fill it.
+constexpr int kTwoPerSM = 2 * 152;
 // M and Q of the grid; false outside the engine (Px < 64).
 bool xg_shape(const Grid& g, int* M, int* Q);
 // Threads and dynamic shared memory of pass 0 (A) or 2 (C); cells: pass C

@@ -126,11 +126,11 @@ int set_up(Setup& S, int nx, int ny, int nz, const double* cell, cudaStream_t s)
     return cudaMemcpyAsync(b + off, src, bytes, cudaMemcpyHostToDevice, s);
   };
   cudaError_t e = cudaSuccess;
-  // the general pass B takes its table in the place of the block engine's (of at least its length)
+  // the general pass B takes its table in the place of the block pass's (of at least its length)
   PassBG bg;
   const bool gen = passb_g_use(g, R, 0) && passb_g_shape(g, &bg);
   // the general passes A and C: their transform table (one class) or the roots
-  // of Px (several) in the place of the block engine's; the transform table of
+  // of Px (several) in the place of the block passes'; the transform table of
   // several classes goes into the build's scratch afterwards
   int xm = 0, xq = 0;
   const bool xg = xg_shape(g, &xm, &xq);

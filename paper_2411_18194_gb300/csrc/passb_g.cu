@@ -47,7 +47,7 @@ PassBGLaunch passb_g_plan(const Grid& g, const PassBG& s, int nplanes) {
   for (int kp = 1; kp <= 8; ++kp) {
     const int gr = (kp * ncol + s.cols - 1) / s.cols;
     if (kp > 1 && (gr > maxw || (size_t)gr * s.cols * s.Q * s.pitch * sizeof(float2) > 64 * 1024)) break;
-    if (kp > 1 && nplanes > 0 && nplanes < kp * 304) break;
+    if (kp > 1 && nplanes > 0 && nplanes < kp * kTwoPerSM) break;
     if (kp > 1 && (kp * ncol) % s.cols != 0 && (ncol % s.cols) == 0) continue;
     l.kp = kp;
     groups = gr;

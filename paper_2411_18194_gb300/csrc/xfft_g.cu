@@ -34,7 +34,7 @@ bool xg_split(const Grid& g, int kind) {
   int M = 0, Q = 0;
   if (!xg_shape(g, &M, &Q) || M <= 8) return false;
   const long long pairs = (long long)((g.ny + 1) / 2) * g.nz;
-  return kind != 0 || (Q > 1 && (g.Px != 2048 || pairs <= 304));
+  return kind != 0 || (Q > 1 && (g.Px != 2048 || pairs <= kTwoPerSM));
 }
 
 // Cells per item of the local field: four, but one or two where that gives a block
@@ -53,7 +53,7 @@ XgPlan xg_plan(const Grid& g, int pass, bool cells, bool batch) {
   int M = 0, Q = 0;
   xg_shape(g, &M, &Q);
   const int warps = M <= 8 ? 1 : 3 * Q;
-  const bool many = batch || (long long)((g.ny + 1) / 2) * g.nz > 304;
+  const bool many = batch || (long long)((g.ny + 1) / 2) * g.nz > kTwoPerSM;
   l.v = many || M > 16 ? 4 : M > 8 ? 2 : 1;
   const int items = pass == 0 ? (g.nx + 1) / 2 : cells ? 2 * g.nx : 2 * g.nx / l.v;
   l.threads = std::max(32 * warps, std::min(many ? 128 : xg_maxthr(Q), (items + 31) / 32 * 32));

@@ -132,7 +132,7 @@ def _make_magnet(w, dt0):
     sh = mag.get_shape()
     ny = w.problem.shape[1]
     if not (sh["engine"] == 3 and _nice(ny) // sh["R"] == 1024):
-        mag.autotune(batch=True)      # cached per geometry: the batch shape (block engine)
+        mag.autotune(batch=True)      # cached per geometry: the batch shape (R = 1, engine 0)
     # else: the warp passes A, B and C (Px = 2048, folded y length 1024), which a
     # batch member runs with launches of its own
     return mag
