@@ -127,8 +127,10 @@ __device__ __forceinline__ void grad3(const float* __restrict__ f, long long n, 
 // about 80 a cell): a cell whose rows are all in the 4th-order bulk takes a path
 // with no selection between them, so that they are in flight together; the
 // selection per term and the 64-bit divisions of the index took most of the time
-// before: 1024x256x1 with two sublattices, cold L2: strain 25 -> 20 us, force 59 -> 38.
-// Antiferromagnet 1024x256x1, four steps (25 launches of each): 4506 -> 3994 us.
+// before.  1024x256x1 with two sublattices, cold L2, us a launch, general form -> bulk
+// path in rows -> packed and by axis: strain 25, 20, 12.5; force 59, 38, 30.5.
+// Antiferromagnet 1024x256x1, four steps (25 launches of each): 2678 -> 2253 us by the
+// last of these.
 // HZ: nz > 1.
 template <bool HZ>
 __global__ void __launch_bounds__(kElThreads) k_strain(Grid g, ElasticArgs e, CellDiv fd, int nsub) {
